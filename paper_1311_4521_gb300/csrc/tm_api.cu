@@ -32,6 +32,31 @@ tm_status cuda_fail(tm_ctx *ctx, cudaError_t e, const char *where)
         if (e_ != cudaSuccess) return cuda_fail(ctx, e_, #call); \
     } while (0)
 
+// Gives an FP64 handle the fixed-point copy of its links (tm_fix.cuh), unless
+// some link does not fit or there is no memory for it: the hops then use
+// FP64 products.  Synchronises s.
+cudaError_t make_fx_links(tm_gauge *h, cudaStream_t s)
+{
+    const size_t bytes = fx_copy_bytes(h);
+    cudaError_t e = cudaMalloc(&h->fx, bytes + sizeof(int));
+    if (e == cudaErrorMemoryAllocation) {
+        (void)cudaGetLastError();   // not sticky: go on without
+        h->fx = nullptr;
+        return cudaSuccess;
+    }
+    if (e != cudaSuccess) return e;
+    int *flag = reinterpret_cast<int *>(static_cast<char *>(h->fx) + bytes), unfit = 0;
+    e = cudaMemsetAsync(flag, 0, sizeof(int), s);
+    if (e == cudaSuccess) e = launch_fx_links(h->geom.vh, h->recon, h->links, h->fx, flag, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&unfit, flag, sizeof(int), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e == cudaSuccess && unfit) {
+        cudaFree(h->fx);
+        h->fx = nullptr;
+    }
+    return e;
+}
+
 bool valid_prec(int p) { return p == TM_F64 || p == TM_F32 || p == TM_F16 || p == TM_F64X; }
 
 }  // namespace
@@ -227,10 +252,10 @@ tm_status tm_gauge_create(tm_ctx *ctx, const int dims[4], const double *U_dev, i
     }
     cudaStream_t s = (cudaStream_t)stream;
     e = launch_pack_gauge(g, prec, reconstruct, U_dev, h->links, s);
+    if (e == cudaSuccess && prec == TM_F64) e = make_fx_links(h, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) {
-        cudaFree(h->links);
-        delete h;
+        tm_gauge_destroy(h);
         return cuda_fail(ctx, e, "tm_gauge_create: pack");
     }
     tm_apply_cached_map(ctx, h);
@@ -242,11 +267,12 @@ void tm_gauge_destroy(tm_gauge *g)
 {
     if (!g) return;
     if (g->links) cudaFree(g->links);
+    if (g->fx) cudaFree(g->fx);
     if (g->links8) cudaFree(g->links8);
     delete g;
 }
 
-size_t tm_gauge_bytes(const tm_gauge *g) { return g ? g->bytes : 0; }
+size_t tm_gauge_bytes(const tm_gauge *g) { return g ? g->bytes + (g->fx ? fx_copy_bytes(g) : 0) : 0; }
 
 tm_status tm_hopping_eo(tm_ctx *ctx, const tm_gauge *U, void *out_dev, const void *in_dev, int dir, int dagger,
                         void *stream)
@@ -255,8 +281,7 @@ tm_status tm_hopping_eo(tm_ctx *ctx, const tm_gauge *U, void *out_dev, const voi
     if (!U || bad_ptr(out_dev) || bad_ptr(in_dev)) return fail(ctx, TM_ERR_ARG, "tm_hopping_eo: null or misaligned pointer");
     if (dir != TM_EO && dir != TM_OE) return fail(ctx, TM_ERR_ARG, "tm_hopping_eo: dir must be TM_EO or TM_OE");
     if (out_dev == in_dev) return fail(ctx, TM_ERR_ARG, "tm_hopping_eo: out and in must not overlap");
-    TM_CUDA(ctx, launch_hop(U->geom, U->prec, U->recon, dagger != 0, dir, U->links, in_dev, out_dev, nullptr,
-                            coef_plain(), (cudaStream_t)stream, U->map));
+    TM_CUDA(ctx, launch_hop(U, dagger != 0, dir, in_dev, out_dev, nullptr, coef_plain(), (cudaStream_t)stream));
     return TM_OK;
 }
 
@@ -268,16 +293,14 @@ tm_status tm_Qtm(tm_ctx *ctx, const tm_gauge *U, void *out_e_dev, const void *in
     if (sign != 1 && sign != -1) return fail(ctx, TM_ERR_ARG, "tm_Qtm: sign must be +1 or -1");
     if (out_e_dev == in_e_dev) return fail(ctx, TM_ERR_ARG, "tm_Qtm: out and in must not overlap");
     void *tmp = nullptr;
-    tm_status st = tm_ctx_scratch(ctx, spinor_bytes(U->geom.vh, U->prec), &tmp);
+    tm_status st = tm_ctx_scratch(ctx, qtm_bytes(U), &tmp);
     if (st != TM_OK) return st;
     double mut = 2.0 * kappa * mu * sign;
     cudaStream_t s = (cudaStream_t)stream;
     tm_trace_mark(ctx, 0, s);
-    TM_CUDA(ctx, launch_hop(U->geom, U->prec, U->recon, false, TM_OE, U->links, in_e_dev, tmp, nullptr,
-                            coef_qtm_a_scaled(kappa, mut), s, U->map));
+    TM_CUDA(ctx, launch_qtm(U, false, false, in_e_dev, tmp, out_e_dev, coef_qtm_a_scaled(kappa, mut), s));
     tm_trace_mark(ctx, 1, s);
-    TM_CUDA(ctx, launch_hop(U->geom, U->prec, U->recon, false, TM_EO, U->links, tmp, out_e_dev, in_e_dev,
-                            coef_qtm_b_unit(mut), s, U->map));
+    TM_CUDA(ctx, launch_qtm(U, false, true, in_e_dev, tmp, out_e_dev, coef_qtm_b_unit(mut), s));
     tm_trace_mark(ctx, 2, s);
     return TM_OK;
 }

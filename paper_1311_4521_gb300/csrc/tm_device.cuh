@@ -61,6 +61,8 @@ enum { F64 = 0, F32 = 1, F16 = 2, F64X = 3 };
 // layout ([site][spin][colour] complex double), read and written in place by
 // the host-field operator (tm_Qtm_host) instead of being packed first.
 enum { F64C = 4 };
+// Nor this one: the library's fixed-point odd temporary (tm_fix.cuh).
+enum { FXF = 5 };
 
 // Conversions between double and the compute type of a storage precision.
 template <typename R> TM_HD R to_R(double x) { return R(x); }
@@ -1023,7 +1025,7 @@ TM_HD void hop_site_src(const Geom &g, const Nbrs &n, const Src &src, const void
         for (int c = 0; c < 3; ++c) acc[s][c] = {R(0), R(0)};
     if constexpr (P == F64X) {
         hop_site_rolled<P, DAG>(g, n, src, in, acc);
-    } else if constexpr (P == F64 || P == F64C) {
+    } else if constexpr (P == F64 || P == F64C || P == FXF) {
         hop_dir_pair<P, DAG, 0, true>(g, n, src, in, acc);
         hop_dir_pair<P, DAG, 1, false>(g, n, src, in, acc);
         hop_dir_pair<P, DAG, 2, false>(g, n, src, in, acc);

@@ -1,0 +1,601 @@
+// tm_fix.cuh -- the FP64 hop with its link products in fixed point.
+//
+// The FP64 units issue 2 lanes per SM and clock here, the integer ones 32
+// lanes of a 32 x 32 -> 64 bit multiply-add (measured: 4.1 cycles per warp
+// and scheduler), and the link multiplies are 576 of the 840 FP64
+// instructions of a site.  So they are done in integers: a hop's projected
+// half-spinor becomes 12 numbers of 58 bits under a common exponent, the
+// links are kept a second time as 58-bit fractions, and a real product is
+// three multiply-adds of 29-bit limbs (the product of the low limbs, below
+// 2^-58 of the largest, is left out).  The 8 hops are summed in 64-bit
+// integers and converted to FP64 once; the epilogue stays in FP64.
+//
+// Precision: a term carries an absolute error of about 2^-57 of the site's
+// largest component, where every FP64 product and sum rounds to 2^-53 of
+// itself; measured against 64-bit and longer arithmetic, Q_tm is off by
+// 1.2e-16 (1.3e-16 with FP64 products).  A site whose neighbours' nonzero
+// components span more than 2^24, or include one that is not finite or near
+// the ends of the exponent range, is computed with FP64 products instead
+// (fx_slow_site), and so is a gauge field with a link outside fx_link_ok.
+//
+// Measured (32^3x64, 18-real links): Q_tm 3.04 -> 0.80 ms, one hop 1.52 ->
+// 0.47 ms; 8^4: Q_tm 65 -> 31 us.  Launch B moves 4.9 TB/s, 0.73 of the
+// measured copy bandwidth; its multiply-add pipe is busy 57 % of the time.
+// What it took beyond the integers (Q_tm at 32^3x64): multiply-adds from
+// plain C, not inline PTX 1.36 -> 1.02 ms; neighbours and links staged by
+// cp.async one hop ahead, 12 warps per SM, 0.87; the fallback called with
+// two words instead of with the site's sum 0.80.
+#pragma once
+
+#include "tm_device.cuh"
+
+namespace twm {
+
+constexpr int FX_LIMB = 29;            // bits of a limb
+constexpr int FX_SPAN = 24;            // log2 of the largest ratio of nonzero components taken here
+constexpr unsigned FX_FMIN = 200, FX_FMAX = 1850;  // biased exponents taken here
+
+// A spinor field of the library's own (the odd temporary of Q_tm) in fixed
+// point: blocks of 32 sites, each 12 arrays of 32 int4 (re.hi, re.lo, im.hi,
+// im.lo) so that a site's loads share one address and differ by constants,
+// then a word per site, (span << 16) + e: component = (hi 2^29 + lo)
+// 2^(e - 57) with the limbs of the component's sign, e the smallest exponent
+// with every |component| < 2^e and span the distance in exponents to the
+// smallest nonzero one.  A site that does not fit holds its FP64 bits and the
+// word FX_RAW.  (One array per component over all sites instead cost two
+// 64-bit additions per load: 3800 against 4400 instructions a site.)
+constexpr int FX_FIELD = 57, FX_HALF = 58;   // fraction bits of field components and of projected half-spinors
+constexpr int FX_RAW = 0x7fffffff, FX_ZERO_E = -4000;
+constexpr unsigned FX_SPINOR_BLOCK = 12 * 32 * 16;
+constexpr unsigned fx_link_block(int recon) { return 4 * (recon / 2) * 32 * 16; }   // 32 sites' links of 4 directions
+TM_HD unsigned fx_blocks(unsigned vh) { return (vh + 31) / 32; }
+TM_HD size_t fx_field_bytes(unsigned vh) { return size_t(FX_SPINOR_BLOCK + 128) * fx_blocks(vh); }
+TM_HD size_t fx_link_bytes(unsigned vh, int recon) { return 2 * size_t(fx_link_block(recon)) * fx_blocks(vh); }
+// Entry of site j in its block (of `block` bytes).
+template <typename T> TM_HD T *fx_entry(T *base, unsigned block, unsigned j)
+{
+    return base + size_t(j >> 5) * (block / unsigned(sizeof(T))) + (j & 31u);
+}
+
+// One link entry as limbs: value = (hi 2^29 + lo) 2^-58, hi and lo of the
+// value's sign; re in x, y and im in z, w.
+typedef int4 FxEntry;
+
+#if defined(__CUDACC__)
+
+// acc + a b, 32 x 32 -> 64 bit: one multiply-add.  (As inline PTX the same
+// sums were compiled to products and separate 64-bit additions: 5683
+// against 3861 instructions a site, 1.36 against 1.02 ms for Q_tm at 32^3x64.)
+__device__ __forceinline__ unsigned long long fx_mad(int a, int b, unsigned long long acc)
+{
+    return acc + (unsigned long long)((long long)a * b);
+}
+// arithmetic shift; amounts above 63 leave the sign
+__device__ __forceinline__ long long fx_sar(long long v, int s)
+{
+    asm("shr.s64 %0, %0, %1;" : "+l"(v) : "r"(s));
+    return v;
+}
+
+// The limbs of v (times -1 if nm is all ones): its mantissa with the leading
+// bit at the top of 64 bits, shifted right by `from` less its biased exponent
+// (and 3 more for the low limb).  The shifts saturate, so zeros and numbers
+// far below the reference vanish.
+__device__ __forceinline__ void fx_split(double v, unsigned from, unsigned nm, int &hi, int &lo)
+{
+    const unsigned hw = unsigned(__double2hiint(v)), lw = unsigned(__double2loint(v));
+    const unsigned th = __funnelshift_l(lw, hw, 11) | 0x80000000u, tl = lw << 11;
+    const unsigned s = from - ((hw >> 20) & 0x7ffu);
+    unsigned mh, ml;
+    asm("shr.u32 %0, %1, %2;" : "=r"(mh) : "r"(th), "r"(s));
+    asm("{ .reg .b64 t; .reg .b32 d; mov.b64 t, {%1, %2}; shr.u64 t, t, %3; mov.b64 {%0, d}, t; }"
+        : "=r"(ml) : "r"(tl), "r"(th), "r"(s + 3u));
+    const int sg = int((unsigned(int(hw) >> 31) ^ nm) | 1u);
+    hi = int(mh) * sg;
+    lo = int(ml & 0x1fffffffu) * sg;
+}
+
+// v 2^(e - bits) in FP64
+__device__ __forceinline__ double fx_to_double(long long v, int e, int bits)
+{
+    const double d = __ll2double_rn(v);
+    const int add = v ? (e - bits) << 20 : 0;
+    return __hiloint2double(__double2hiint(d) + add, __double2loint(d));
+}
+
+__device__ __forceinline__ const int *fx_words(const void *base, unsigned vh)
+{
+    return reinterpret_cast<const int *>(static_cast<const char *>(base) + size_t(FX_SPINOR_BLOCK) * fx_blocks(vh));
+}
+
+// Fixed-point fields read and written as FP64 sites.
+template <> struct SpinorIO<FXF> {
+    using R = double;
+    __device__ static R load_raw(const void *base, unsigned vh, unsigned i, Spinor<R> &s)
+    {
+        const int4 *b = fx_entry(static_cast<const int4 *>(base), FX_SPINOR_BLOCK, i);
+        const int word = fx_words(base, vh)[i];
+        const int e = int(short(word & 0xffff));
+#pragma unroll
+        for (int c = 0; c < 12; ++c) {
+            const int4 v = b[32 * c];
+            if (word == FX_RAW)
+                s[c / 3][c % 3] = {__hiloint2double(v.x, v.y), __hiloint2double(v.z, v.w)};
+            else
+                s[c / 3][c % 3] = {fx_to_double(((long long)v.x << FX_LIMB) + v.y, e, FX_FIELD),
+                                   fx_to_double(((long long)v.z << FX_LIMB) + v.w, e, FX_FIELD)};
+        }
+        return R(1);
+    }
+    __device__ __forceinline__ static void store(void *base, unsigned vh, unsigned i, const Spinor<R> &s)
+    {
+        int4 *b = fx_entry(static_cast<int4 *>(base), FX_SPINOR_BLOCK, i);
+        unsigned m = 0, lowest = 0xffffffffu;   // of the high words without sign; zeros wrap and do not count
+        unsigned bits = 0;
+#pragma unroll
+        for (int c = 0; c < 12; ++c) {
+            const cpx<R> v = s[c / 3][c % 3];
+            const unsigned p = unsigned(__double2hiint(v.re)) & 0x7fffffffu, q = unsigned(__double2hiint(v.im)) & 0x7fffffffu;
+            m = max(m, max(p, q));
+            lowest = min(lowest, min(p - 1u, q - 1u));
+            bits |= p | q | unsigned(__double2loint(v.re)) | unsigned(__double2loint(v.im));
+        }
+        const bool zero = bits == 0;
+        const unsigned f = m >> 20;
+        const unsigned span = zero ? 0u : f - ((lowest + 1u) >> 20);
+        const bool raw = !zero && (f < FX_FMIN || f > FX_FMAX || span > unsigned(FX_SPAN));
+        const int e = zero ? FX_ZERO_E : int(f) - 1022;
+        const unsigned from = zero ? 8000u : f + 4u;
+#pragma unroll
+        for (int c = 0; c < 12; ++c) {
+            const cpx<R> v = s[c / 3][c % 3];
+            int4 o;
+            fx_split(v.re, from, 0u, o.x, o.y);
+            fx_split(v.im, from, 0u, o.z, o.w);
+            if (raw) o = make_int4(__double2hiint(v.re), __double2loint(v.re), __double2hiint(v.im), __double2loint(v.im));
+            st_stream(b + 32 * c, o);
+        }
+        st_stream(const_cast<int *>(fx_words(base, vh)) + i, raw ? FX_RAW : int(span << 16) | (e & 0xffff));
+    }
+};
+
+// A site's sum: 64-bit integers in units of 2^(e - bits).
+struct FxSum {
+    long long re[4][3], im[4][3];
+    int e;
+};
+
+// A projected half-spinor as limbs (in units that the sum's exponent fixes).
+struct FxHalf {
+    int hi[2][3][2], lo[2][3][2];
+};
+
+// Adds (r, S A_mu^dag r) for one component r of the upper spin s: the lower
+// spin that it feeds, times +-1 or +-i, as in accumulate().
+template <int MU, int S> __device__ __forceinline__ void fx_accumulate(int s, int c, long long re, long long im, FxSum &t)
+{
+    t.re[s][c] += re;
+    t.im[s][c] += im;
+    // lower spin 2 + k and its factor: MU 0: -s h_k; 1: s i h_(1-k); 2: s h1, -s h0; 3: s i h0, -s i h1
+    const int k = (MU == 0 || MU == 3) ? s : 1 - s;
+    const bool times_i = MU == 1 || MU == 3;
+    bool minus = S < 0;
+    if (MU == 0) minus = !minus;
+    if (MU == 2 && s == 0) minus = !minus;
+    if (MU == 3 && s == 1) minus = !minus;
+    const long long a = times_i ? im : re, b = times_i ? re : im;   // i r = (-im, re)
+    if (minus != times_i) t.re[2 + k][c] -= a;
+    else t.re[2 + k][c] += a;
+    if (minus) t.im[2 + k][c] -= b;
+    else t.im[2 + k][c] += b;
+}
+
+// The fixed-point links: per origin parity blocks of 32 sites, each with one
+// FxEntry array of 32 for every direction and stored complex entry.
+template <int RECON> struct FxLinks {
+    const FxEntry *links;
+    unsigned vh, i;
+    int p;
+    template <int MU, bool FWD> __device__ __forceinline__ const FxEntry *at(const Nbrs &n) const
+    {
+        constexpr unsigned blk = fx_link_block(RECON);
+        const FxEntry *b = links + size_t(FWD ? p : 1 - p) * fx_blocks(vh) * (blk / 16);
+        return fx_entry(b, blk, FWD ? i : n.bwd[MU]) + MU * (RECON / 2) * 32;
+    }
+};
+
+// One component of conj(row0 x row1): conj(a d - b c), as limbs.
+__device__ __forceinline__ FxEntry fx_minor(const FxEntry &a, const FxEntry &d, const FxEntry &b, const FxEntry &c)
+{
+    unsigned long long hr = 0, mr = 0, hi = 0, mi = 0;
+    // re = a.re d.re - a.im d.im - b.re c.re + b.im c.im ; im = -(a.re d.im + a.im d.re - b.re c.im - b.im c.re)
+    auto put = [](int xh, int xl, int yh, int yl, unsigned long long &h, unsigned long long &m) {
+        h = fx_mad(xh, yh, h);
+        m = fx_mad(xh, yl, m);
+        m = fx_mad(xl, yh, m);
+    };
+    put(a.x, a.y, d.x, d.y, hr, mr);
+    put(-a.z, -a.w, d.z, d.w, hr, mr);
+    put(-b.x, -b.y, c.x, c.y, hr, mr);
+    put(b.z, b.w, c.z, c.w, hr, mr);
+    put(-a.x, -a.y, d.z, d.w, hi, mi);
+    put(-a.z, -a.w, d.x, d.y, hi, mi);
+    put(b.x, b.y, c.z, c.w, hi, mi);
+    put(b.z, b.w, c.x, c.y, hi, mi);
+    const long long re = (long long)hr + ((long long)mr >> FX_LIMB), im = (long long)hi + ((long long)mi >> FX_LIMB);
+    FxEntry r;
+    r.x = int(re >> FX_LIMB);
+    r.y = int(re & ((1 << FX_LIMB) - 1));
+    r.z = int(im >> FX_LIMB);
+    r.w = int(im & ((1 << FX_LIMB) - 1));
+    return r;
+}
+
+// Whether a link (as limbs, each component below 1 + 2^-20) can be used: every
+// row's and column's sum of |re| + |im| at most 2.5 (sqrt(6) bounds it for a
+// unitary matrix), which bounds the sum of the 8 hops by 8 * 2.5 * 2^59 <
+// 2^63, and its largest component at least 1/16 (or all of them zero).
+__device__ __forceinline__ bool fx_link_ok(const FxEntry (&u)[9])
+{
+    constexpr int most = int(2.5 * (1 << FX_LIMB));   // limbs are below 2^30, so three entries sum below 2^32.6
+    bool ok = true;
+    unsigned bits = 0;
+    int big = 0;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        unsigned row = 0, col = 0;
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+            const FxEntry r = u[3 * a + b], c = u[3 * b + a];
+            row += unsigned(abs(r.x) + abs(r.z)) >> 1;
+            col += unsigned(abs(c.x) + abs(c.z)) >> 1;
+            big = max(big, max(abs(r.x), abs(r.z)));
+            bits |= unsigned(r.x | r.y | r.z | r.w);
+        }
+        ok = ok && row <= unsigned(most) / 2 && col <= unsigned(most) / 2;
+    }
+    return ok && (big >= 1 << (FX_LIMB - 4) || bits == 0);
+}
+
+// Staging of a hop's data: every thread copies its own neighbour site (12
+// 16-byte words) and link (RECON / 2 words) to its own slots of shared
+// memory with cp.async, one hop ahead of the arithmetic, so that the loads
+// in flight take no registers and no thread waits for another.  The site's
+// words are read into registers (projected) before the next hop's copies
+// start, so they need one slot; the links need two.
+constexpr int FX_BLOCK = 64;   // threads per CTA of the fixed-point hops
+template <int RECON> struct FxStage {
+    static constexpr int NL = RECON / 2, WORDS = 12 + 2 * NL;
+    int4 *slot;   // this thread's first word; word w at slot[w * FX_BLOCK]
+    __device__ __forceinline__ int4 spinor(int c) const { return slot[c * FX_BLOCK]; }
+    // the staged FP64 site
+    __device__ __forceinline__ void site(Spinor<double> &s) const
+    {
+#pragma unroll
+        for (int c = 0; c < 12; ++c) {
+            const int4 v = spinor(c);
+            s[c / 3][c % 3] = {__hiloint2double(v.y, v.x), __hiloint2double(v.w, v.z)};
+        }
+    }
+    __device__ __forceinline__ int4 link(int q, int k) const { return slot[(12 + q * NL + k) * FX_BLOCK]; }
+    __device__ __forceinline__ void copy(int w, const void *src) const
+    {
+        const unsigned dst = unsigned(__cvta_generic_to_shared(slot + w * FX_BLOCK));
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+    }
+    // Starts the copies of one hop, the link into slot q: the words of the
+    // site at s (sstride apart) and of the link at u.
+    __device__ __forceinline__ void start(int q, const int4 *s, size_t sstride, const FxEntry *u) const
+    {
+#pragma unroll
+        for (int c = 0; c < 12; ++c) copy(c, s + c * sstride);
+#pragma unroll
+        for (int k = 0; k < NL; ++k) copy(12 + q * NL + k, u + 32 * k);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    __device__ __forceinline__ void start_site(const int4 *s, size_t sstride) const
+    {
+#pragma unroll
+        for (int c = 0; c < 12; ++c) copy(c, s + c * sstride);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    __device__ __forceinline__ void wait() const { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
+};
+
+// The link product of direction MU on x, aligned to the sum by a right shift
+// of d, added to the sum.  A 32 x 32 -> 64 bit multiply-add takes 4 issue
+// cycles of a scheduler, an addition 2 on another pipe, so complex products
+// use three real ones: with w = ur + ui (ur - ui for the conjugate link of a
+// backward hop) and K = w hr,
+//     re = K -+ ui (hr + hi),   im = K + ur (hi - hr).
+// Per sum the products with one low limb come first; shifted by a limb they
+// join the sum of the high ones.  Intermediate sums may wrap, results do not.
+template <int MU, int S, bool FWD, bool ALIGN, int RECON>
+__device__ __forceinline__ void fx_apply(const FxStage<RECON> &st, int q, const FxHalf &x, int d, FxSum &t)
+{
+    int sh[2][3], sl[2][3], dh[2][3], dl[2][3];   // -+(hr + hi) and hi - hr
+#pragma unroll
+    for (int s = 0; s < 2; ++s)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            sh[s][c] = FWD ? -x.hi[s][c][0] - x.hi[s][c][1] : x.hi[s][c][0] + x.hi[s][c][1];
+            sl[s][c] = FWD ? -x.lo[s][c][0] - x.lo[s][c][1] : x.lo[s][c][0] + x.lo[s][c][1];
+            dh[s][c] = x.hi[s][c][1] - x.hi[s][c][0];
+            dl[s][c] = x.lo[s][c][1] - x.lo[s][c][0];
+        }
+    FxEntry full[RECON == 12 ? 9 : 1];
+    if constexpr (RECON == 12) {
+#pragma unroll
+        for (int k = 0; k < 6; ++k) full[k] = st.link(q, k);
+        full[6] = fx_minor(full[1], full[5], full[2], full[4]);
+        full[7] = fx_minor(full[2], full[3], full[0], full[5]);
+        full[8] = fx_minor(full[0], full[4], full[1], full[3]);
+    }
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        FxEntry u[3];
+        int wh[3], wl[3];
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+            const int k = FWD ? 3 * a + b : 3 * b + a;
+            u[b] = RECON == 12 ? full[RECON == 12 ? k : 0] : st.link(q, k);
+            wh[b] = FWD ? u[b].x + u[b].z : u[b].x - u[b].z;
+            wl[b] = FWD ? u[b].y + u[b].w : u[b].y - u[b].w;
+        }
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+            unsigned long long k = 0, re, im;
+#pragma unroll
+            for (int b = 0; b < 3; ++b) {
+                k = fx_mad(wh[b], x.lo[s][b][0], k);
+                k = fx_mad(wl[b], x.hi[s][b][0], k);
+            }
+            re = im = k;
+#pragma unroll
+            for (int b = 0; b < 3; ++b) {
+                re = fx_mad(u[b].z, sl[s][b], re);
+                im = fx_mad(u[b].x, dl[s][b], im);
+                re = fx_mad(u[b].w, sh[s][b], re);
+                im = fx_mad(u[b].y, dh[s][b], im);
+            }
+            k = 0;
+#pragma unroll
+            for (int b = 0; b < 3; ++b) k = fx_mad(wh[b], x.hi[s][b][0], k);
+            re = k + ((long long)re >> FX_LIMB);
+            im = k + ((long long)im >> FX_LIMB);
+#pragma unroll
+            for (int b = 0; b < 3; ++b) {
+                re = fx_mad(u[b].z, sh[s][b], re);
+                im = fx_mad(u[b].x, dh[s][b], im);
+            }
+            long long r = (long long)re, i = (long long)im;
+            if (ALIGN) {
+                r = fx_sar(r, d);
+                i = fx_sar(i, d);
+            }
+            fx_accumulate<MU, S>(s, a, r, i, t);
+        }
+    }
+}
+
+// ---- input in fixed point (FXF)
+// The projected half-spinor of the fixed-point site j: project() on limbs.
+template <int MU, int S, class Stage> __device__ __forceinline__ void fx_project(const Stage &st, FxHalf &x)
+{
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        int4 p[4];
+#pragma unroll
+        for (int s = 0; s < 4; ++s) p[s] = st.spinor(3 * s + c);
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+            // h_s = u_s + S (A_mu l)_s: the lower spin and its factor (1 or i, signed)
+            const int4 l = p[2 + ((MU == 0 || MU == 3) ? s : 1 - s)];
+            const bool times_i = MU == 1 || MU == 3;
+            bool minus = S < 0;
+            if (MU == 0 || MU == 1) minus = !minus;           // A_0 l = -l; A_1 l = (-i l1, -i l0)
+            if (MU == 2 && s == 0) minus = !minus;            // A_2 l = (-l1, l0)
+            if (MU == 3 && s == 0) minus = !minus;            // A_3 l = (-i l0, i l1)
+            const int rh = times_i ? -l.z : l.x, rl = times_i ? -l.w : l.y;
+            const int ih = times_i ? l.x : l.z, il = times_i ? l.y : l.w;
+            x.hi[s][c][0] = minus ? p[s].x - rh : p[s].x + rh;
+            x.lo[s][c][0] = minus ? p[s].y - rl : p[s].y + rl;
+            x.hi[s][c][1] = minus ? p[s].z - ih : p[s].z + ih;
+            x.lo[s][c][1] = minus ? p[s].w - il : p[s].w + il;
+        }
+    }
+}
+
+__device__ __forceinline__ void fx_negate(FxHalf &x, int sg)
+{
+#pragma unroll
+    for (int s = 0; s < 2; ++s)
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                x.hi[s][c][k] *= sg;
+                x.lo[s][c][k] *= sg;
+            }
+}
+
+// ---- input in FP64
+// h (times -1 if neg) as limbs of 58 bits under the sum's exponent, which is
+// raised (to one more than h needs) where h does not fit.
+struct FxRange {
+    unsigned fmax = 0, fmin = 0xffffffffu;   // high words met without sign; fmin less one, so that zeros do not count
+    bool bad = false;
+};
+__device__ __forceinline__ void fx_from_half(const Half<double> &h, bool neg, FxHalf &x, FxSum &t, FxRange &q)
+{
+    unsigned m = 0, lowest = 0xffffffffu;
+#pragma unroll
+    for (int s = 0; s < 2; ++s)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const unsigned a = unsigned(__double2hiint(h[s][c].re)) & 0x7fffffffu;
+            const unsigned b = unsigned(__double2hiint(h[s][c].im)) & 0x7fffffffu;
+            m = max(m, max(a, b));
+            lowest = min(lowest, min(a - 1u, b - 1u));
+        }
+    const int e = int(m >> 20) - 1022;   // |h| < 2^e
+    if (m < (FX_FMIN << 20)) {           // all zero, or too small for the integer path
+#pragma unroll
+        for (int s = 0; s < 2; ++s)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) q.bad = q.bad || h[s][c].re != 0.0 || h[s][c].im != 0.0;
+    } else {
+        q.fmax = max(q.fmax, m);
+        q.fmin = min(q.fmin, lowest);
+        if (e > t.e) {
+            const int s = e + 1 - t.e;
+#pragma unroll
+            for (int sp = 0; sp < 4; ++sp)
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    t.re[sp][c] = fx_sar(t.re[sp][c], s);
+                    t.im[sp][c] = fx_sar(t.im[sp][c], s);
+                }
+            t.e = e + 1;
+        }
+    }
+    const unsigned from = unsigned(t.e + 1022 + 3), nm = neg ? 0xffffffffu : 0u;
+#pragma unroll
+    for (int s = 0; s < 2; ++s)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            fx_split(h[s][c].re, from, nm, x.hi[s][c][0], x.lo[s][c][0]);
+            fx_split(h[s][c].im, from, nm, x.hi[s][c][1], x.lo[s][c][1]);
+        }
+}
+
+// ---- the 8 hops
+// Starts the copies of hop K (2 mu, or 2 mu + 1 for the backward one).
+template <int P, int K, int RECON>
+__device__ __forceinline__ void fx_start(const Geom &g, const Nbrs &n, const FxLinks<RECON> &src, const void *in, const FxStage<RECON> &st)
+{
+    constexpr int MU = K >> 1;
+    const unsigned j = K & 1 ? n.bwd[MU] : n.fwd[MU];
+    const int4 *f = static_cast<const int4 *>(in);
+    const FxEntry *u = src.template at<MU, !(K & 1)>(n);
+    if (P == FXF) st.start(K & 1, fx_entry(f, FX_SPINOR_BLOCK, j), 32, u);
+    else if (P == F64C) st.start(K & 1, f + size_t(j) * 12, 1, u);
+    else st.start(K & 1, f + j, g.vh, u);
+}
+
+// Hop K and those after it.  SIGNS: whether directions other than time may
+// have a boundary sign.
+template <int P, bool DAG, int K, bool SIGNS, int RECON>
+__device__ __forceinline__ void fx_hops(const Geom &g, const Nbrs &n, const FxLinks<RECON> &src, const void *in,
+                                        const FxStage<RECON> &st, const int4 *x0, size_t xstride, unsigned long long d,
+                                        FxSum &t, FxRange &r)
+{
+    st.wait();
+    constexpr int MU = K >> 1, q = K & 1;
+    constexpr int S = (DAG ? +1 : -1) * (q ? -1 : 1);
+    const bool neg = (MU == 0 || SIGNS) && (q ? n.wb[MU] : n.wf[MU]) && g.anti[MU];
+    FxHalf x;
+    if constexpr (P == FXF) {
+        fx_project<MU, S>(st, x);
+        if (MU == 0 || SIGNS) fx_negate(x, neg ? -1 : 1);
+    } else {
+        Spinor<double> s;
+        Half<double> h;
+        st.site(s);
+        project<MU, S>(s, h);
+        fx_from_half(h, neg, x, t, r);
+    }
+    __syncwarp();   // the site's words are read before the next copies start
+    if constexpr (K < 7) fx_start<P, K + 1>(g, n, src, in, st);
+    else if (x0) st.start_site(x0, xstride);
+    fx_apply<MU, S, q == 0, P == FXF, RECON>(st, q, x, int(unsigned(d >> (8 * K)) & 0xffu), t);
+    if constexpr (K < 7) fx_hops<P, DAG, K + 1, SIGNS>(g, n, src, in, st, x0, xstride, d, t, r);
+}
+
+// Everything a fixed-point hop launch needs; a kernel parameter that device
+// functions read in place.
+struct FxArgs {
+    Geom g;
+    SiteMap m;
+    Coef k;
+    int p;                  // output parity
+    const FxEntry *fx;      // fixed-point links
+    const double2 *links;   // FP64 links
+    const void *in, *x;
+    void *out;
+};
+
+// Output site i with FP64 products, from the input to the stored result: for
+// the few sites that the integer path does not take.  A call whose arguments
+// are two words: passing the site's sum in and out cost 7 % of the kernel.
+template <int PI, int PX, int PO, int RECON, bool DAG, bool HASX>
+__device__ __noinline__ void fx_slow_site(const FxArgs &A, unsigned i)
+{
+    Nbrs n;
+    neighbours(A.g, A.p, i, n);
+    GlobalLinks<F64, RECON> src{A.links, A.g.vh, i, A.p};
+    Spinor<double> acc, xs, o;
+    hop_site_src<PI, DAG>(A.g, n, src, A.in, acc);
+    if (HASX) SpinorIO<PX>::load(A.x, A.g.vh, i, xs);
+    epilogue(A.k, acc, HASX ? &xs : nullptr, o);
+    SpinorIO<PO>::store(A.out, A.g.vh, i, o);
+}
+
+// The hop at output site i; every thread of the warp calls it.  Returns
+// whether the site is one that the integer path does not take (acc is not
+// its hop then).  With x0 set, the 12 words at x0, xstride apart, are in the
+// stage's site slot on return.
+template <int P, int RECON, bool DAG, bool SIGNS>
+__device__ __forceinline__ bool fx_hop_site(const FxArgs &A, unsigned i, const FxStage<RECON> &st, const int4 *x0,
+                                            size_t xstride, Spinor<double> &acc)
+{
+    const Geom &g = A.g;
+    const void *in = A.in;
+    Nbrs n;
+    neighbours(g, A.p, i, n);
+    const FxLinks<RECON> src{A.fx, g.vh, i, A.p};
+    fx_start<P, 0>(g, n, src, in, st);
+    FxSum t;
+#pragma unroll
+    for (int s = 0; s < 4; ++s)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) t.re[s][c] = t.im[s][c] = 0;
+    FxRange r;
+    unsigned long long d = 0;   // per hop a byte: the shift that aligns it to the site's exponent
+    t.e = P == FXF ? FX_ZERO_E : -5000;
+    bool slow = false;
+    if constexpr (P == FXF) {
+        const int *word = fx_words(in, g.vh);
+        int e[8], low = 0x7fff;
+#pragma unroll
+        for (int m = 0; m < 8; ++m) e[m] = ld_keep(word + (m & 1 ? n.bwd[m >> 1] : n.fwd[m >> 1]));
+#pragma unroll
+        for (int m = 0; m < 8; ++m) {
+            slow = slow || e[m] == FX_RAW;
+            const int span = e[m] >> 16;
+            e[m] = int(short(e[m] & 0xffff));
+            t.e = max(t.e, e[m]);
+            low = min(low, e[m] == FX_ZERO_E ? 0x7fff : e[m] - span);
+        }
+        slow = slow || t.e - low > FX_SPAN;
+#pragma unroll
+        for (int m = 0; m < 8; ++m) d |= (unsigned long long)(unsigned(min(t.e - e[m], 63))) << (8 * m);
+    }
+    fx_hops<P, DAG, 0, SIGNS>(g, n, src, in, st, x0, xstride, d, t, r);
+    if constexpr (P != FXF) {
+        const unsigned top = r.fmax >> 20, low = (r.fmin + 1u) >> 20;
+        slow = r.bad || top > FX_FMAX || (r.fmax && top - low > unsigned(FX_SPAN));
+    }
+    if (slow) return true;
+    constexpr int bits = P == FXF ? FX_FIELD : FX_HALF;
+#pragma unroll
+    for (int s = 0; s < 4; ++s)
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+            acc[s][c] = {fx_to_double(t.re[s][c], t.e, bits), fx_to_double(t.im[s][c], t.e, bits)};
+    return false;
+}
+
+#endif  // __CUDACC__
+
+}  // namespace twm

@@ -218,12 +218,12 @@ extern "C" tm_status tm_force_ex(tm_ctx *ctx, const tm_gauge *U, double *F_dev, 
     const double mut = 2.0 * kappa * mu;
     cudaStream_t s = (cudaStream_t)stream;
     // Z = M_oo^-1 H_oe X, Y = Q X, B = gamma5 (M_oo^-1)^dag H_oe Y
-    cudaError_t e = launch_hop(U->geom, U->prec, U->recon, false, TM_OE, U->links, X_e_dev, Zo, nullptr,
-                               coef_qtm_a(mut), s, U->map);
+    cudaError_t e = launch_hop(U, false, TM_OE, X_e_dev, Zo, nullptr,
+                               coef_qtm_a(mut), s);
     if (e == cudaSuccess)
-        e = launch_hop(U->geom, U->prec, U->recon, false, TM_EO, U->links, Zo, Ye, X_e_dev, coef_qtm_b(kappa, mut), s, U->map);
+        e = launch_hop(U, false, TM_EO, Zo, Ye, X_e_dev, coef_qtm_b(kappa, mut), s);
     if (e == cudaSuccess)
-        e = launch_hop(U->geom, U->prec, U->recon, false, TM_OE, U->links, Ye, Bo, nullptr, coef_force_b(mut), s, U->map);
+        e = launch_hop(U, false, TM_OE, Ye, Bo, nullptr, coef_force_b(mut), s);
     const double k2 = kappa * kappa;
     if (e == cudaSuccess && scheme == TM_FORCE_OWNER) {
         switch (U->prec * 100 + U->recon) {
@@ -296,10 +296,9 @@ extern "C" tm_status tm_link_grad(tm_ctx *ctx, const tm_gauge *U, double *G_dev,
     cudaError_t e = cudaSuccess;
     if (op == TM_GRAD_QTM) {
         const double mut = 2.0 * kappa * mu * sign;
-        e = launch_hop(U->geom, U->prec, U->recon, false, TM_OE, U->links, X_dev, w0, nullptr, coef_qtm_a(mut), s, U->map);
+        e = launch_hop(U, false, TM_OE, X_dev, w0, nullptr, coef_qtm_a(mut), s);
         if (e == cudaSuccess)
-            e = launch_hop(U->geom, U->prec, U->recon, false, TM_OE, U->links, Y_dev, w1, nullptr, coef_force_b(mut), s,
-                           U->map);
+            e = launch_hop(U, false, TM_OE, Y_dev, w1, nullptr, coef_force_b(mut), s);
         Xe = X_dev, Ye = Y_dev, Zo = w0, Bo = w1;
         k2 = -0.5 * kappa * kappa;
     } else if (op == TM_GRAD_HOP_EO) {

@@ -104,6 +104,7 @@ struct tm_gauge {
     size_t bytes = 0;
     twm::SiteMap map{};   // site-to-thread map of this lattice's hop launches (tm_gauge_tune)
     std::string map_name = "linear128";
+    void *fx = nullptr;   // FP64 handles whose links fit (tm_fix.cuh): their fixed-point copy
     mutable void *links8 = nullptr;  // site-complete link copy of the staged batched hop (built on first use)
 };
 
@@ -120,21 +121,38 @@ void tune_cache_store(const std::string &path, const std::string &key, const std
 
 namespace twm {
 
+// The FP64 hop with fixed-point link products (tm_fix.cu), for handles with
+// a fixed-point link copy: making that copy (*unfit, device memory, is set
+// where a link cannot be used), the hop on FP64 fields, and the two stages
+// of Q_tm on packed or canonical FP64 fields with the odd temporary in fixed
+// point; tmp holds fx_qtm_bytes.
+cudaError_t launch_fx_links(unsigned vh, int recon, const void *links, void *fx, int *unfit, cudaStream_t s);
+cudaError_t launch_fx_hop(const tm_gauge *U, bool dag, int out_parity, const void *in, void *out, const void *x,
+                          const Coef &k, cudaStream_t s, const SiteMap &m);
+size_t fx_copy_bytes(const tm_gauge *U);
+size_t fx_qtm_bytes(unsigned vh);
+cudaError_t launch_fx_qtm(const tm_gauge *U, bool canonical, bool stage_b, const void *in, void *tmp, void *out,
+                          const Coef &k, cudaStream_t s);
+
 // Fills the geometry of a lattice; returns false if the extents are invalid.
 bool make_geom(const int dims[4], const int bc[4], Geom &g);
 
+// The two stages of Q_tm and their odd temporary (the scratch of qtm_bytes):
+// stage A in -> tmp, stage B tmp -> out with in re-read.  canonical: FP64
+// fields in the caller's canonical layout.
+size_t qtm_bytes(const tm_gauge *U);
+cudaError_t launch_qtm(const tm_gauge *U, bool canonical, bool stage_b, const void *in, void *tmp, void *out,
+                       const Coef &k, cudaStream_t s);
+
 // Launchers (tm_kernels.cu).  All enqueue on `s` and return the launch status.
-// Q_tm of an FP64 handle on fields in the canonical layout: launch A
-// (in_can -> tmp, an odd packed FP64 field) or launch B (tmp -> out_can,
-// in_can re-read), with coefficients k.
-cudaError_t launch_qtm_canonical(bool stage_b, const Geom &g, int recon, const SiteMap &m, const void *links,
-                                 const double *in_can, void *tmp, double *out_can, const Coef &k, cudaStream_t s);
-// The hop with the given site-to-thread map, or with the linear map of
-// `block` threads per CTA.
-cudaError_t launch_hop(const Geom &g, int prec, int recon, bool dag, int out_parity, const void *links,
-                       const void *in, void *out, const void *x, const Coef &k, cudaStream_t s, const SiteMap &m);
-cudaError_t launch_hop(const Geom &g, int prec, int recon, bool dag, int out_parity, const void *links,
-                       const void *in, void *out, const void *x, const Coef &k, cudaStream_t s, int block);
+// The hop of U's lattice with its site-to-thread map (or the map m).
+cudaError_t launch_hop(const tm_gauge *U, bool dag, int out_parity, const void *in, void *out, const void *x,
+                       const Coef &k, cudaStream_t s, const SiteMap &m);
+inline cudaError_t launch_hop(const tm_gauge *U, bool dag, int out_parity, const void *in, void *out, const void *x,
+                              const Coef &k, cudaStream_t s)
+{
+    return launch_hop(U, dag, out_parity, in, out, x, k, s, U->map);
+}
 cudaError_t launch_pack_gauge(const Geom &g, int prec, int recon, const double *U, void *links, cudaStream_t s);
 cudaError_t launch_pack_spinor(unsigned vh, int prec, const double *in, void *out, cudaStream_t s);
 cudaError_t launch_unpack_spinor(unsigned vh, int prec, const void *in, double *out, cudaStream_t s);

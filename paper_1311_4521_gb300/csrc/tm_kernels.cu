@@ -111,24 +111,30 @@ __global__ void __launch_bounds__(128, TM_HOP_MINB(F64))
 }
 
 template <int RECON>
-static cudaError_t qtm_canonical(bool stage_b, const Geom &g, const SiteMap &m, const void *links,
-                                 const double *in_can, void *tmp, double *out_can, const Coef &k, cudaStream_t s)
+static cudaError_t qtm_canonical(bool stage_b, const Geom &g, const SiteMap &m, const void *links, const void *in,
+                                 void *tmp, void *out, const Coef &k, cudaStream_t s)
 {
     using V = typename LinkIO<F64, RECON>::V;
     const V *l = static_cast<const V *>(links);
     const unsigned grid = map_grid(g, m);
-    if (!stage_b) k_hop_io<F64C, F64, F64, RECON, false><<<grid, m.block, 0, s>>>(g, 1, l, in_can, tmp, nullptr, k, m);
-    else k_hop_io<F64, F64C, F64C, RECON, true><<<grid, m.block, 0, s>>>(g, 0, l, tmp, out_can, in_can, k, m);
+    if (!stage_b) k_hop_io<F64C, F64, F64, RECON, false><<<grid, m.block, 0, s>>>(g, 1, l, in, tmp, nullptr, k, m);
+    else k_hop_io<F64, F64C, F64C, RECON, true><<<grid, m.block, 0, s>>>(g, 0, l, tmp, out, in, k, m);
     return cudaGetLastError();
 }
 
-cudaError_t launch_qtm_canonical(bool stage_b, const Geom &g, int recon, const SiteMap &m, const void *links,
-                                 const double *in_can, void *tmp, double *out_can, const Coef &k, cudaStream_t s)
+size_t qtm_bytes(const tm_gauge *U) { return U->fx ? fx_qtm_bytes(U->geom.vh) : spinor_bytes(U->geom.vh, U->prec); }
+
+cudaError_t launch_qtm(const tm_gauge *U, bool canonical, bool stage_b, const void *in, void *tmp, void *out,
+                       const Coef &k, cudaStream_t s)
 {
+    const Geom &g = U->geom;
     if (g.vh == 0) return cudaSuccess;
-    if (recon == 18) return qtm_canonical<18>(stage_b, g, m, links, in_can, tmp, out_can, k, s);
-    if (recon == 12) return qtm_canonical<12>(stage_b, g, m, links, in_can, tmp, out_can, k, s);
-    return cudaErrorInvalidValue;
+    if (U->fx) return launch_fx_qtm(U, canonical, stage_b, in, tmp, out, k, s);
+    if (!canonical) {
+        return stage_b ? launch_hop(U, false, TM_EO, tmp, out, in, k, s) : launch_hop(U, false, TM_OE, in, tmp, nullptr, k, s);
+    }
+    if (U->recon == 18) return qtm_canonical<18>(stage_b, g, U->map, U->links, in, tmp, out, k, s);
+    return qtm_canonical<12>(stage_b, g, U->map, U->links, in, tmp, out, k, s);
 }
 
 template <int P, int RECON>
@@ -144,24 +150,23 @@ static cudaError_t hop_dispatch(const Geom &g, bool dag, int p, const void *link
     return cudaGetLastError();
 }
 
-cudaError_t launch_hop(const Geom &g, int prec, int recon, bool dag, int out_parity, const void *links,
-                       const void *in, void *out, const void *x, const Coef &k, cudaStream_t s, const SiteMap &m)
+cudaError_t launch_hop(const tm_gauge *U, bool dag, int out_parity, const void *in, void *out, const void *x,
+                       const Coef &k, cudaStream_t s, const SiteMap &m)
 {
+    const Geom &g = U->geom;
     if (g.vh == 0) return cudaSuccess;
-    if (prec == F64 && recon == 18) return hop_dispatch<F64, 18>(g, dag, out_parity, links, in, out, x, k, s, m);
-    if (prec == F64 && recon == 12) return hop_dispatch<F64, 12>(g, dag, out_parity, links, in, out, x, k, s, m);
-    if (prec == F32 && recon == 18) return hop_dispatch<F32, 18>(g, dag, out_parity, links, in, out, x, k, s, m);
-    if (prec == F32 && recon == 12) return hop_dispatch<F32, 12>(g, dag, out_parity, links, in, out, x, k, s, m);
-    if (prec == F16 && recon == 12) return hop_dispatch<F16, 12>(g, dag, out_parity, links, in, out, x, k, s, m);
-    if (prec == F64X && recon == 18) return hop_dispatch<F64X, 18>(g, dag, out_parity, links, in, out, x, k, s, m);
-    if (prec == F64X && recon == 12) return hop_dispatch<F64X, 12>(g, dag, out_parity, links, in, out, x, k, s, m);
+    if (U->fx) return launch_fx_hop(U, dag, out_parity, in, out, x, k, s, m);
+    const void *l = U->links;
+    switch (U->prec * 100 + U->recon) {
+    case F64 * 100 + 18: return hop_dispatch<F64, 18>(g, dag, out_parity, l, in, out, x, k, s, m);
+    case F64 * 100 + 12: return hop_dispatch<F64, 12>(g, dag, out_parity, l, in, out, x, k, s, m);
+    case F32 * 100 + 18: return hop_dispatch<F32, 18>(g, dag, out_parity, l, in, out, x, k, s, m);
+    case F32 * 100 + 12: return hop_dispatch<F32, 12>(g, dag, out_parity, l, in, out, x, k, s, m);
+    case F16 * 100 + 12: return hop_dispatch<F16, 12>(g, dag, out_parity, l, in, out, x, k, s, m);
+    case F64X * 100 + 18: return hop_dispatch<F64X, 18>(g, dag, out_parity, l, in, out, x, k, s, m);
+    case F64X * 100 + 12: return hop_dispatch<F64X, 12>(g, dag, out_parity, l, in, out, x, k, s, m);
+    }
     return cudaErrorInvalidValue;
-}
-
-cudaError_t launch_hop(const Geom &g, int prec, int recon, bool dag, int out_parity, const void *links,
-                       const void *in, void *out, const void *x, const Coef &k, cudaStream_t s, int block)
-{
-    return launch_hop(g, prec, recon, dag, out_parity, links, in, out, x, k, s, linear_map(unsigned(block)));
 }
 
 // ------------------------------------------------------------------ layouts

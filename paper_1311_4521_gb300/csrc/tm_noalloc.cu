@@ -89,12 +89,12 @@ extern "C" tm_status tm_Qtm_noalloc(tm_ctx *ctx, const tm_gauge *U, void *out_e_
     double mut = 2.0 * kappa * mu * sign;
     cudaStream_t s = (cudaStream_t)stream;
     tm_trace_mark(ctx, 0, s);
-    cudaError_t e = launch_hop(U->geom, U->prec, U->recon, false, TM_OE, U->links, in_e_dev, tmp, nullptr,
-                               coef_qtm_a_scaled(kappa, mut), s, 128);
+    cudaError_t e = launch_hop(U, false, TM_OE, in_e_dev, tmp, nullptr,
+                               coef_qtm_a_scaled(kappa, mut), s, linear_map(128));
     if (e == cudaSuccess) {
         tm_trace_mark(ctx, 1, s);
-        e = launch_hop(U->geom, U->prec, U->recon, false, TM_EO, U->links, tmp, out_e_dev, in_e_dev,
-                       coef_qtm_b_unit(mut), s, 128);
+        e = launch_hop(U, false, TM_EO, tmp, out_e_dev, in_e_dev,
+                       coef_qtm_b_unit(mut), s, linear_map(128));
     }
     if (e == cudaSuccess) tm_trace_mark(ctx, 2, s);
     if (e != cudaSuccess)

@@ -129,11 +129,11 @@ float time_map(const tm_gauge *U, const SiteMap &m, const void *in, void *out, c
     cudaEvent_t ev[4];
     for (auto &e : ev) cudaEventCreate(&e);
     const Coef k = coef_qtm_b_unit(0.01);
-    err = launch_hop(U->geom, U->prec, U->recon, false, TM_EO, U->links, in, out, x, k, s, m);
+    err = launch_hop(U, false, TM_EO, in, out, x, k, s, m);
     cudaEventRecord(ev[0], s);
     for (int r = 0; r < 3 && err == cudaSuccess; ++r) {
         for (int q = 0; q < 2 && err == cudaSuccess; ++q)
-            err = launch_hop(U->geom, U->prec, U->recon, false, TM_EO, U->links, in, out, x, k, s, m);
+            err = launch_hop(U, false, TM_EO, in, out, x, k, s, m);
         cudaEventRecord(ev[r + 1], s);
     }
     float ms[3] = {1e30f, 1e30f, 1e30f};
