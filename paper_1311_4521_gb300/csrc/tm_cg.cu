@@ -18,66 +18,13 @@
 #include <cstdio>
 #include <cstring>
 
-#include "tm_cg.cuh"
+#include "tm_cg_fix.cuh"
 #include "tm_internal.h"
 
 namespace twm {
 
-// Block sum of v; the block's partial goes to partials[blockIdx.x] and the
-// last block to arrive sums all partials in index order and finishes `op`.
-// Every thread of the block must call this.
-template <int BLOCK>
-__device__ void reduce_finish(double v, double *partials, CgScalars *s, int op)
-{
-    __shared__ double sh[BLOCK / 32];
-    __shared__ bool last;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    if (lane == 0) sh[warp] = v;
-    __syncthreads();
-    if (warp == 0) {
-        v = lane < BLOCK / 32 ? sh[lane] : 0.0;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-        if (lane == 0) {
-            partials[blockIdx.x] = v;
-            __threadfence();
-            unsigned t = atomicAdd(&s->ticket, 1u);
-            last = (t == gridDim.x - 1);
-        }
-    }
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-    double acc = 0.0;
-    const volatile double *vp = partials;
-    for (unsigned k = threadIdx.x; k < gridDim.x; k += BLOCK) acc += vp[k];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-    __syncthreads();
-    if (lane == 0) sh[warp] = acc;
-    __syncthreads();
-    if (warp == 0) {
-        acc = lane < BLOCK / 32 ? sh[lane] : 0.0;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-        if (lane == 0) {
-            cg_finish(op, acc, s);
-            s->ticket = 0;
-        }
-    }
-}
-
 constexpr int HOP_BLOCK = 128;
 constexpr int LA_BLOCK = 256;
-
-// Hop with the twisted-mass epilogue.  MODE HOP_NORM also reduces |out|^2
-// into pAp; MODE HOP_UPDATE is the last hop of Q^dag Q p: instead of storing
-// its result Ap it applies the CG update at once, y += alpha p and
-// r -= alpha Ap (y in precision PY), and reduces |r|^2 into rr_new, so Ap is
-// never written to memory and read back.
-enum { HOP_PLAIN = 0, HOP_NORM = 1, HOP_UPDATE = 2 };
 
 template <int P, int RECON, int MODE>
 __global__ void __launch_bounds__(HOP_BLOCK, TM_HOP_MINB(P)) k_cg_hop(Geom g, int p, const typename LinkIO<P, RECON>::V *__restrict__ links,
@@ -132,9 +79,10 @@ __global__ void __launch_bounds__(HOP_BLOCK, TM_HOP_MINB(P)) k_cg_hop(Geom g, in
 }
 
 // p = r + beta p with beta = rr_new / rr (restart: p = r); then rr = rr_new.
+// p_fx (may be null, P = F64): a fixed-point copy of p for the next hop.
 template <int P>
 __global__ void __launch_bounds__(LA_BLOCK, (P == F64 || P == F64X) ? 3 : 4) k_cg_pupdate(unsigned vh, void *p, const void *r, double *partials,
-                                                         CgScalars *s, int skip, int restart)
+                                                         CgScalars *s, int skip, int restart, void *p_fx)
 {
     using R = typename SpinorIO<P>::R;
     if (skip && s->done) return;
@@ -155,6 +103,8 @@ __global__ void __launch_bounds__(LA_BLOCK, (P == F64 || P == F64X) ? 3 : 4) k_c
                 }
         }
         SpinorIO<P>::store(p, vh, i, rv);
+        if constexpr (P == F64)
+            if (p_fx) SpinorIO<FXF>::store(p_fx, vh, i, rv);
     }
     reduce_finish<LA_BLOCK>(0.0, partials, s, FIN_ROLL);
 }
@@ -259,6 +209,7 @@ struct Work {
     void *x, *b, *ax, *t_hi, *q_hi, *r_hi;
     // inner fields (precision P), y in PY
     void *r, *p, *q, *t, *y;
+    void *p_fx;         // fixed-point copy of p (FP64 solver on a handle with fixed-point links), else null
     double *partials;
     CgScalars *s;
 };
@@ -301,6 +252,17 @@ cudaError_t qdagq(const tm_gauge *U, double kappa, double mu, const void *in, vo
                   bool iterate, const Work &w, int gate, cudaStream_t st)
 {
     double mut = 2.0 * kappa * mu;
+    if (U->fx) {   // t and q in fixed point
+        const CgFxArgs c{static_cast<double *>(w.y), static_cast<double *>(w.r), w.p, w.partials, w.s, gate};
+        cudaError_t e = cudaSuccess;
+        for (int stage = 0; stage < 4 && e == cudaSuccess; ++stage) {
+            const double m = stage < 2 ? mut : -mut;
+            const Coef k = stage & 1 ? coef_qtm_b_unit(m) : coef_qtm_a_scaled(kappa, m);
+            e = (U->recon == 18 ? cg_fx_stage_18 : cg_fx_stage_12)(U, stage, in, iterate ? w.p_fx : nullptr, t, q,
+                                                                   iterate ? w.ax : out, iterate, k, c, st);
+        }
+        return e;
+    }
     cudaError_t e = hop(U, 1, in, t, nullptr, coef_qtm_a_scaled(kappa, mut), HOP_PLAIN, w, gate, st);
     if (e == cudaSuccess) e = hop(U, 0, t, q, in, coef_qtm_b_unit(mut), iterate ? HOP_NORM : HOP_PLAIN, w, gate, st);
     if (e == cudaSuccess) e = hop(U, 1, q, t, nullptr, coef_qtm_a_scaled(kappa, -mut), HOP_PLAIN, w, gate, st);
@@ -311,10 +273,10 @@ cudaError_t qdagq(const tm_gauge *U, double kappa, double mu, const void *in, vo
 cudaError_t pupdate(const Work &w, int skip, int restart, cudaStream_t st)
 {
     unsigned g = blocks(w.vh, LA_BLOCK);
-    if (w.P == F64) k_cg_pupdate<F64><<<g, LA_BLOCK, 0, st>>>(w.vh, w.p, w.r, w.partials, w.s, skip, restart);
-    else if (w.P == F64X) k_cg_pupdate<F64X><<<g, LA_BLOCK, 0, st>>>(w.vh, w.p, w.r, w.partials, w.s, skip, restart);
-    else if (w.P == F32) k_cg_pupdate<F32><<<g, LA_BLOCK, 0, st>>>(w.vh, w.p, w.r, w.partials, w.s, skip, restart);
-    else k_cg_pupdate<F16><<<g, LA_BLOCK, 0, st>>>(w.vh, w.p, w.r, w.partials, w.s, skip, restart);
+    if (w.P == F64) k_cg_pupdate<F64><<<g, LA_BLOCK, 0, st>>>(w.vh, w.p, w.r, w.partials, w.s, skip, restart, w.p_fx);
+    else if (w.P == F64X) k_cg_pupdate<F64X><<<g, LA_BLOCK, 0, st>>>(w.vh, w.p, w.r, w.partials, w.s, skip, restart, w.p_fx);
+    else if (w.P == F32) k_cg_pupdate<F32><<<g, LA_BLOCK, 0, st>>>(w.vh, w.p, w.r, w.partials, w.s, skip, restart, w.p_fx);
+    else k_cg_pupdate<F16><<<g, LA_BLOCK, 0, st>>>(w.vh, w.p, w.r, w.partials, w.s, skip, restart, w.p_fx);
     return cudaGetLastError();
 }
 
@@ -451,9 +413,13 @@ extern "C" tm_status tm_cg_QdagQ(tm_ctx *ctx, const tm_gauge *U_hi, const tm_gau
     if (!w.mixed) S.Ul = U_hi;
 
     // workspace: FP64 ax, t_hi, q_hi (+ r in plain mode), inner r, p, q, t, y, partials, scalars
+    // (the hop temporaries t, q in fixed point where the handle has fixed-point links)
+    const bool fx_lo = S.Ul->fx != nullptr;
     const size_t f64 = spinor_bytes(w.vh, w.PH), flo = spinor_bytes(w.vh, w.P), fy = spinor_bytes(w.vh, w.PY);
-    const size_t nblk = blocks(w.vh, 128) + 1;
-    size_t need = 3 * align256(f64) + 4 * align256(flo) + (w.mixed ? align256(fy) : 0) + align256(nblk * sizeof(double)) + align256(sizeof(CgScalars));
+    const size_t ffx = fx_field_bytes(w.vh), tq_hi = U_hi->fx ? ffx : f64, tq = fx_lo ? ffx : flo;
+    const size_t nblk = blocks(w.vh, FX_BLOCK) + 1;   // the smallest CTA of a reducing launch
+    size_t need = align256(f64) + 2 * align256(tq_hi) + 2 * align256(flo) + 2 * align256(tq) + (fx_lo ? align256(ffx) : 0) +
+                  (w.mixed ? align256(fy) : 0) + align256(nblk * sizeof(double)) + align256(sizeof(CgScalars));
     void *base = nullptr;
     tm_status st = tm_ctx_workspace(ctx, need, &base);
     if (st != TM_OK) return st;
@@ -462,12 +428,13 @@ extern "C" tm_status tm_cg_QdagQ(tm_ctx *ctx, const tm_gauge *U_hi, const tm_gau
     w.x = x_dev;
     w.b = const_cast<void *>(b_dev);
     w.ax = take(f64);
-    w.t_hi = take(f64);
-    w.q_hi = take(f64);
+    w.t_hi = take(tq_hi);
+    w.q_hi = take(tq_hi);
     w.r = take(flo);
     w.p = take(flo);
-    w.q = take(flo);
-    w.t = take(flo);
+    w.q = take(tq);
+    w.t = take(tq);
+    w.p_fx = fx_lo ? take(ffx) : nullptr;
     w.y = w.mixed ? take(fy) : x_dev;   // plain FP64: the update adds straight into x
     w.r_hi = w.r;
     w.partials = static_cast<double *>(take(nblk * sizeof(double)));

@@ -112,5 +112,57 @@ template <typename R> __device__ __forceinline__ double norm2(const Spinor<R> &a
     return double(n);
 }
 
+// Block sum of v; the block's partial goes to partials[blockIdx.x] and the
+// last block to arrive sums all partials in index order and finishes `op`.
+// Every thread of the block must call this.
+template <int BLOCK>
+__device__ void reduce_finish(double v, double *partials, CgScalars *s, int op)
+{
+    __shared__ double sh[BLOCK / 32];
+    __shared__ bool last;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    if (lane == 0) sh[warp] = v;
+    __syncthreads();
+    if (warp == 0) {
+        v = lane < BLOCK / 32 ? sh[lane] : 0.0;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+        if (lane == 0) {
+            partials[blockIdx.x] = v;
+            __threadfence();
+            unsigned t = atomicAdd(&s->ticket, 1u);
+            last = (t == gridDim.x - 1);
+        }
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    double acc = 0.0;
+#pragma unroll 8
+    for (unsigned k = threadIdx.x; k < gridDim.x; k += BLOCK) acc += __ldcg(partials + k);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+    __syncthreads();
+    if (lane == 0) sh[warp] = acc;
+    __syncthreads();
+    if (warp == 0) {
+        acc = lane < BLOCK / 32 ? sh[lane] : 0.0;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+        if (lane == 0) {
+            cg_finish(op, acc, s);
+            s->ticket = 0;
+        }
+    }
+}
+
+// Hop with the twisted-mass epilogue.  MODE HOP_NORM also reduces |out|^2
+// into pAp; MODE HOP_UPDATE is the last hop of Q^dag Q p: instead of storing
+// its result Ap it applies the CG update at once, y += alpha p and
+// r -= alpha Ap (y in precision PY), and reduces |r|^2 into rr_new, so Ap is
+// never written to memory and read back.
+enum { HOP_PLAIN = 0, HOP_NORM = 1, HOP_UPDATE = 2 };
 
 }  // namespace twm

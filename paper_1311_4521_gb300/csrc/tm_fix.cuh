@@ -127,6 +127,7 @@ template <> struct SpinorIO<FXF> {
         }
         return R(1);
     }
+    __device__ static void load(const void *base, unsigned vh, unsigned i, Spinor<R> &s) { load_raw(base, vh, i, s); }
     __device__ __forceinline__ static void store(void *base, unsigned vh, unsigned i, const Spinor<R> &s)
     {
         int4 *b = fx_entry(static_cast<int4 *>(base), FX_SPINOR_BLOCK, i);
