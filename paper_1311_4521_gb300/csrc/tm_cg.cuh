@@ -31,6 +31,10 @@ struct CgScalars {
     int mixed;       // 1: reduced-precision inner solver with reliable updates
     int nreliable;   // FP64 residual recomputations so far
     unsigned ticket; // last-block-done counter of the current reduction
+    // graph replay (zero without): the handles of the loop over iterations and
+    // of the reliable update inside it, iterations of the current segment
+    unsigned long long loop, update;
+    int segment, loops;
 };
 
 // Gates of the iteration kernels: 0 always run, 1 skip once the solve is
@@ -38,6 +42,17 @@ struct CgScalars {
 __device__ __forceinline__ bool gated(const CgScalars *s, int gate)
 {
     return gate == 1 ? s->done != 0 : gate == 2 ? s->reliable == 0 : false;
+}
+
+// The end of an iteration: whether the graph's loop runs another one.  Every
+// path of an iteration's last kernel comes here, so a segment ends after at
+// most `segment` iterations.
+__device__ __forceinline__ void cg_loop_end(CgScalars *s)
+{
+    if (!s->loop) return;
+    const bool more = !s->done && ++s->loops < s->segment;
+    if (!more) s->loops = 0;
+    cudaGraphSetConditional(s->loop, more);
 }
 
 enum Fin { FIN_PAP, FIN_RR_UPDATE, FIN_RR_TRUE, FIN_RR_CHECK, FIN_BB, FIN_ROLL };
@@ -69,6 +84,7 @@ __device__ __forceinline__ void cg_finish(int op, double total, CgScalars *s)
         } else if (stop) {
             s->pending = 1;
         }
+        if (s->update) cudaGraphSetConditional(s->update, s->reliable != 0);
         break;
     }
     case FIN_RR_TRUE:
@@ -94,6 +110,7 @@ __device__ __forceinline__ void cg_finish(int op, double total, CgScalars *s)
             s->done = 1;
             s->pending = 0;
         }
+        cg_loop_end(s);
         break;
     }
     if (bad && op != FIN_ROLL) {
