@@ -183,6 +183,9 @@ tm_status tm_spinor_unpack(tm_ctx *ctx, long vh, const void *in_dev, double *out
  * and keeps no reference to U_dev.  Synchronous with respect to stream. */
 tm_status tm_gauge_create(tm_ctx *ctx, const int dims[4], const double *U_dev, int prec, int reconstruct,
                           const int bc[4], void *stream, tm_gauge **out);
+/* The context keeps the link buffers of the last destroyed handles (at most
+ * two, together at most 1 GiB) for the next handles that fit, until it and
+ * its last handle are destroyed.  A handle may outlive its context. */
 void tm_gauge_destroy(tm_gauge *g);
 /* Bytes of device memory held by the handle's link storage.  A TM_F64 handle
  * also holds, memory permitting, a fixed-point copy of its links of the same
@@ -433,8 +436,8 @@ tm_status tm_force_ex(tm_ctx *ctx, const tm_gauge *U, double *F_dev, const void 
  * and odd temporaries are owned by ctx.  Asynchronous on `stream` like
  * tm_Qtm: the first call for a batch (its handles, field pointers, lattice
  * sizes and stream) uploads its tables and, for a new batch shape, times
- * launch configurations (both synchronise the stream); a repeated call with
- * the same batch only launches.  Batched calls on one ctx that overlap on
+ * launch configurations (which synchronises the stream); a repeated call
+ * with the same batch only launches.  Batched calls on one ctx that overlap on
  * different streams are not supported (the ctx synchronises the previous
  * stream when the stream changes). */
 tm_status tm_Qtm_batch(tm_ctx *ctx, int nsys, const tm_gauge *const *U, void *const *out_e, const void *const *in_e,

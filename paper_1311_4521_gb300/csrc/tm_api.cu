@@ -32,28 +32,17 @@ tm_status cuda_fail(tm_ctx *ctx, cudaError_t e, const char *where)
         if (e_ != cudaSuccess) return cuda_fail(ctx, e_, #call); \
     } while (0)
 
-// Gives an FP64 handle the fixed-point copy of its links (tm_fix.cuh), unless
-// some link does not fit or there is no memory for it: the hops then use
-// FP64 products.  Synchronises s.
-cudaError_t make_fx_links(tm_gauge *h, cudaStream_t s)
+// Makes the fixed-point copy of an FP64 handle's links (tm_fix.cuh) in the
+// fx_copy_bytes + sizeof(int) bytes at fx; the handle keeps it unless some
+// link does not fit (the hops then use FP64 products).  Synchronises s.
+cudaError_t make_fx_links(tm_gauge *h, void *fx, cudaStream_t s)
 {
-    const size_t bytes = fx_copy_bytes(h);
-    cudaError_t e = cudaMalloc(&h->fx, bytes + sizeof(int));
-    if (e == cudaErrorMemoryAllocation) {
-        (void)cudaGetLastError();   // not sticky: go on without
-        h->fx = nullptr;
-        return cudaSuccess;
-    }
-    if (e != cudaSuccess) return e;
-    int *flag = reinterpret_cast<int *>(static_cast<char *>(h->fx) + bytes), unfit = 0;
-    e = cudaMemsetAsync(flag, 0, sizeof(int), s);
-    if (e == cudaSuccess) e = launch_fx_links(h->geom.vh, h->recon, h->links, h->fx, flag, s);
+    int *flag = reinterpret_cast<int *>(static_cast<char *>(fx) + fx_copy_bytes(h)), unfit = 0;
+    cudaError_t e = cudaMemsetAsync(flag, 0, sizeof(int), s);
+    if (e == cudaSuccess) e = launch_fx_links(h->geom.vh, h->recon, h->links, fx, flag, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(&unfit, flag, sizeof(int), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e == cudaSuccess && unfit) {
-        cudaFree(h->fx);
-        h->fx = nullptr;
-    }
+    if (e == cudaSuccess && !unfit) h->fx = fx;
     return e;
 }
 
@@ -91,6 +80,62 @@ tm_status tm_ctx_reduce_buffer(tm_ctx *ctx, size_t bytes, void **ptr)
     }
     *ptr = ctx->red;
     return TM_OK;
+}
+
+cudaError_t LinkPool::take(size_t bytes, void **p, size_t *size)
+{
+    {
+        std::lock_guard<std::mutex> guard(lock_);
+        for (size_t k = 0; k < spare_.size(); ++k) {
+            if (spare_[k].second < bytes || spare_[k].second > 2 * bytes) continue;
+            *p = spare_[k].first;
+            *size = spare_[k].second;
+            spare_.erase(spare_.begin() + long(k));
+            const cudaError_t e = cudaDeviceSynchronize();
+            if (e != cudaSuccess) {
+                cudaFree(*p);
+                *p = nullptr;
+            }
+            return e;
+        }
+    }
+    cudaError_t e = cudaMalloc(p, bytes);
+    if (e == cudaErrorMemoryAllocation) {
+        (void)cudaGetLastError();   // not sticky
+        trim();
+        e = cudaMalloc(p, bytes);
+        if (e == cudaErrorMemoryAllocation) (void)cudaGetLastError();
+    }
+    *size = e == cudaSuccess ? bytes : 0;
+    return e;
+}
+
+void LinkPool::give(void *p, size_t size)
+{
+    std::vector<void *> drop;
+    {
+        std::lock_guard<std::mutex> guard(lock_);
+        if (size > kMost) {
+            drop.push_back(p);
+        } else {
+            size_t total = size;
+            for (auto &b : spare_) total += b.second;
+            while (!spare_.empty() && (spare_.size() >= 2 || total > kMost)) {   // the oldest go first
+                total -= spare_.front().second;
+                drop.push_back(spare_.front().first);
+                spare_.erase(spare_.begin());
+            }
+            spare_.push_back({p, size});
+        }
+    }
+    for (void *q : drop) cudaFree(q);
+}
+
+void LinkPool::trim()
+{
+    std::lock_guard<std::mutex> guard(lock_);
+    for (auto &b : spare_) cudaFree(b.first);
+    spare_.clear();
 }
 
 extern "C" {
@@ -245,14 +290,19 @@ tm_status tm_gauge_create(tm_ctx *ctx, const int dims[4], const double *U_dev, i
     h->recon = reconstruct;
     h->geom = g;
     h->bytes = size_t(8) * link_nchunk(prec, reconstruct) * link_chunk_bytes(prec, reconstruct) * g.vh;
-    cudaError_t e = cudaMalloc(&h->links, h->bytes);
+    h->pool = ctx->pool;
+    // the links, and for FP64 handles room for their fixed-point copy where there is memory
+    const size_t own = align256(h->bytes), copy = prec == TM_F64 ? fx_copy_bytes(h) + sizeof(int) : 0;
+    cudaError_t e = h->pool->take(own + copy, &h->links, &h->links_size);
+    const bool room = e == cudaSuccess;
+    if (e == cudaErrorMemoryAllocation && copy) e = h->pool->take(own, &h->links, &h->links_size);
     if (e != cudaSuccess) {
         delete h;
         return cuda_fail(ctx, e, "cudaMalloc(links)");
     }
     cudaStream_t s = (cudaStream_t)stream;
     e = launch_pack_gauge(g, prec, reconstruct, U_dev, h->links, s);
-    if (e == cudaSuccess && prec == TM_F64) e = make_fx_links(h, s);
+    if (e == cudaSuccess && copy && room) e = make_fx_links(h, static_cast<char *>(h->links) + own, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) {
         tm_gauge_destroy(h);
@@ -266,8 +316,7 @@ tm_status tm_gauge_create(tm_ctx *ctx, const int dims[4], const double *U_dev, i
 void tm_gauge_destroy(tm_gauge *g)
 {
     if (!g) return;
-    if (g->links) cudaFree(g->links);
-    if (g->fx) cudaFree(g->fx);
+    if (g->links) g->pool->give(g->links, g->links_size);
     if (g->links8) cudaFree(g->links8);
     delete g;
 }

@@ -299,7 +299,8 @@ int zband_for(const Geom &g, unsigned ts)
 // launches differ by less than their spread), so the order is fixed per format.
 bool band_order(int prec) { return prec != F16; }
 
-// Fills a hop table for pass width nrb and uploads it to `dev` (capacity ngroups).
+// Fills a hop table for pass width nrb and uploads it to `dev` (capacity
+// ngroups).  The copy from pageable memory has taken the data when it returns.
 cudaError_t build_table(const std::vector<BGroup> &tmpl, int nrb, unsigned grid_cap, HopTable &t, BGroup *dev,
                         cudaStream_t st, std::vector<BGroup> &host, const StageArgs &sa = StageArgs{},
                         bool band = true)
@@ -379,17 +380,16 @@ cudaError_t tune_hop_table(tm_ctx *ctx, int prec, int recon, const std::vector<B
         const std::vector<int> ok = nrb_candidates(prec, recon, std::max(nrhs_max, 2), sa != nullptr);
         if (std::find(ok.begin(), ok.end(), ctx->batch_code) != ok.end()) {
             const unsigned dcap = ctx->batch_code == STAGE_CODE ? sms : 1u << 30;
-            cudaError_t e = build_table(tmpl, ctx->batch_code, ctx->batch_cap ? ctx->batch_cap : dcap, out, dev,
-                                        st, host, sta, band_order(prec));
-            if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-            return e;
+            return build_table(tmpl, ctx->batch_code, ctx->batch_cap ? ctx->batch_cap : dcap, out, dev, st, host, sta,
+                               band_order(prec));
         }
     }
     if (sa) key += "/staged";
     auto it = ctx->tuned.find(key);
     // a choice persisted by an earlier process (tm_ctx_set_tune_cache), if its code is a candidate here
-    const std::string ckey = tune_cache_gpu(ctx) + "|" + key;
-    if (it == ctx->tuned.end() && ctx->autotune && !ctx->tune_cache.empty()) {
+    const bool cache = it == ctx->tuned.end() && ctx->autotune && !ctx->tune_cache.empty();
+    const std::string ckey = cache ? tune_cache_gpu(ctx) + "|" + key : "";   // a device query: only where it is used
+    if (cache) {
         std::string val;
         double cms = 0;
         int code = -1;
@@ -404,12 +404,8 @@ cudaError_t tune_hop_table(tm_ctx *ctx, int prec, int recon, const std::vector<B
             }
         }
     }
-    if (it != ctx->tuned.end()) {
-        cudaError_t e = build_table(tmpl, it->second.first, it->second.second, out, dev, st, host, sta,
-                                    band_order(prec));
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-        return e;
-    }
+    if (it != ctx->tuned.end())
+        return build_table(tmpl, it->second.first, it->second.second, out, dev, st, host, sta, band_order(prec));
     float best = 1e30f;
     int best_nrb = 1;
     unsigned best_cap = 1u << 30;
@@ -438,7 +434,7 @@ cudaError_t tune_hop_table(tm_ctx *ctx, int prec, int recon, const std::vector<B
     ctx->tuned[key] = {best_nrb, best_cap};
     ctx->tuned_ms[key] = best;
     ctx->tuned_band[key] = band_order(prec) ? 1 : 0;
-    if (ctx->autotune && !ctx->tune_cache.empty())
+    if (cache)
         tune_cache_store(ctx->tune_cache, ckey, "code" + std::to_string(best_nrb) + "-cap" + std::to_string(best_cap),
                          best);
     cudaError_t e = build_table(tmpl, best_nrb, best_cap, out, dev, st, host, sta, band_order(prec));
@@ -509,10 +505,15 @@ extern "C" tm_status tm_Qtm_batch(tm_ctx *ctx, int nsys, const tm_gauge *const *
         if (bad_ptr(out_e[k]) || bad_ptr(in_e[k]) || out_e[k] == in_e[k]) return tm_fail(ctx, TM_ERR_ARG, "tm_Qtm_batch: bad field pointer");
     }
     {   // every output is written by one system and read by none (inputs may repeat)
-        std::set<const void *> outs(out_e, out_e + nsys), ins(in_e, in_e + nsys);
-        if (int(outs.size()) != nsys) return tm_fail(ctx, TM_ERR_ARG, "tm_Qtm_batch: an output field appears twice");
-        for (const void *o : outs)
-            if (ins.count(o)) return tm_fail(ctx, TM_ERR_ARG, "tm_Qtm_batch: an output field is also an input");
+        std::vector<uintptr_t> outs(nsys), ins(nsys);
+        for (int k = 0; k < nsys; ++k) outs[k] = uintptr_t(out_e[k]), ins[k] = uintptr_t(in_e[k]);
+        std::sort(outs.begin(), outs.end());
+        std::sort(ins.begin(), ins.end());
+        if (std::adjacent_find(outs.begin(), outs.end()) != outs.end())
+            return tm_fail(ctx, TM_ERR_ARG, "tm_Qtm_batch: an output field appears twice");
+        for (uintptr_t o : outs)
+            if (std::binary_search(ins.begin(), ins.end(), o))
+                return tm_fail(ctx, TM_ERR_ARG, "tm_Qtm_batch: an output field is also an input");
     }
     cudaStream_t s = (cudaStream_t)stream;
     // The staged hop is a candidate where every lattice is tiled by its boxes

@@ -245,7 +245,8 @@ def tm_ctx_tune_report(ctx) -> str:
 
 
 def _parr(items):
-    return (ctypes.c_void_p * len(items))(*[(_ptr(t).value or 0) if not isinstance(t, ctypes.c_void_p) else t.value
+    return (ctypes.c_void_p * len(items))(*[t.data_ptr() if isinstance(t, torch.Tensor) else
+                                            t.value if isinstance(t, ctypes.c_void_p) else int(t) if t is not None else 0
                                             for t in items])
 
 
