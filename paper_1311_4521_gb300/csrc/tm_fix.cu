@@ -101,17 +101,162 @@ __global__ void __launch_bounds__(FX_BLOCK, TM_FX_MINB)
     SpinorIO<PO>::store(A.out, g.vh, i, o);
 }
 
-static unsigned fx_grid(unsigned vh) { return (vh + FX_BLOCK - 1) / FX_BLOCK; }
+// The same hop with the 8 hops of a site dealt out to four warps, one
+// direction each, for lattices whose sites do not fill the GPU: a CTA covers
+// 32 sites.  The warps' integer sums meet in shared memory, then warp w
+// finishes spin w.  The site map is not used (results do not depend on it).
+constexpr int FX_SPLIT = 128;
+template <int RECON> constexpr size_t fx_split_bytes() { return sizeof(int4) * FxStage<RECON, FX_SPLIT>::WORDS * FX_SPLIT; }
+
+template <int PI, int PX, int PO, int RECON, bool DAG, bool HASX, bool SIGNS>
+__global__ void __launch_bounds__(FX_SPLIT, 3) k_fx_hop_split(const __grid_constant__ FxArgs A)
+{
+    extern __shared__ int4 dyn[];
+    __shared__ int4 info[FX_SPLIT];
+    const Geom &g = A.g;
+    const unsigned vh = g.vh, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const unsigned site = blockIdx.x * 32 + lane, i = min(site, vh - 1);
+    const FxStage<RECON, FX_SPLIT> st{dyn + threadIdx.x};
+    Nbrs n;
+    neighbours(g, A.p, i, n);
+    const FxLinks<RECON> src{A.fx, vh, i, A.p};
+    FxSum t;
+#pragma unroll
+    for (int s = 0; s < 4; ++s)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) t.re[s][c] = t.im[s][c] = 0;
+    FxRange r;
+    unsigned long long d = 0;
+    t.e = -5000;
+    switch (w) {
+    case 0: fx_start<PI, 0>(g, n, src, A.in, st); break;
+    case 1: fx_start<PI, 2>(g, n, src, A.in, st); break;
+    case 2: fx_start<PI, 4>(g, n, src, A.in, st); break;
+    default: fx_start<PI, 6>(g, n, src, A.in, st);
+    }
+    double2 x[3];   // spin w of the re-read input
+    if (HASX)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const double2 *b = static_cast<const double2 *>(A.x);
+            x[c] = ld_keep(PX == F64C ? b + size_t(i) * 12 + 3 * w + c : b + size_t(3 * w + c) * vh + i);
+        }
+    bool slow = false;
+    if constexpr (PI == FXF) slow = fx_exponents(n, A.in, vh, t.e, d);
+    switch (w) {
+    case 0: fx_hops<PI, DAG, 0, 1, SIGNS>(g, n, src, A.in, st, nullptr, 0, d, t, r); break;
+    case 1: fx_hops<PI, DAG, 2, 3, SIGNS>(g, n, src, A.in, st, nullptr, 0, d, t, r); break;
+    case 2: fx_hops<PI, DAG, 4, 5, SIGNS>(g, n, src, A.in, st, nullptr, 0, d, t, r); break;
+    default: fx_hops<PI, DAG, 6, 7, SIGNS>(g, n, src, A.in, st, nullptr, 0, d, t, r);
+    }
+    if constexpr (PI != FXF) {   // the directions' exponents and ranges meet first
+        info[threadIdx.x] = make_int4(t.e, int(r.fmax), int(r.fmin), r.bad);
+        __syncthreads();
+        const int own = t.e;
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            const int4 q = info[32 * v + lane];
+            t.e = max(t.e, q.x);
+            r.fmax = max(r.fmax, unsigned(q.y));
+            r.fmin = min(r.fmin, unsigned(q.z));
+            r.bad = r.bad || q.w;
+        }
+        slow = fx_range_slow(r);
+#pragma unroll
+        for (int s = 0; s < 4; ++s)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                t.re[s][c] = fx_sar(t.re[s][c], t.e - own);
+                t.im[s][c] = fx_sar(t.im[s][c], t.e - own);
+            }
+    } else {
+        __syncthreads();   // every warp has read its staged words
+    }
+    long long *part = reinterpret_cast<long long *>(dyn);   // [24][4 directions][32]
+#pragma unroll
+    for (int s = 0; s < 4; ++s)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            part[(6 * s + 2 * c) * FX_SPLIT + threadIdx.x] = t.re[s][c];
+            part[(6 * s + 2 * c + 1) * FX_SPLIT + threadIdx.x] = t.im[s][c];
+        }
+    __syncthreads();
+    constexpr int bits = PI == FXF ? FX_FIELD : FX_HALF;
+    const bool up = w < 2;
+    const cpx<double> a = up ? cpx<double>{A.k.d[0], A.k.d[1]} : cpx<double>{A.k.d[2], A.k.d[3]};
+    const cpx<double> b = up ? cpx<double>{A.k.d[4], A.k.d[5]} : cpx<double>{A.k.d[6], A.k.d[7]};
+    cpx<double> o[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const long long *q = part + (6 * w + 2 * c) * FX_SPLIT + lane;
+        const long long re = q[0] + q[32] + q[64] + q[96];
+        const long long im = q[FX_SPLIT] + q[FX_SPLIT + 32] + q[FX_SPLIT + 64] + q[FX_SPLIT + 96];
+        const cpx<double> hop = {fx_to_double(re, t.e, bits), fx_to_double(im, t.e, bits)};
+        o[c] = A.k.unit ? (up ? hop : -hop) : a * hop;
+        if (HASX) o[c] = cmadd(b, cpx<double>{x[c].x, x[c].y}, o[c]);
+    }
+    if constexpr (PO == FXF) {
+        unsigned m = 0, lowest = 0xffffffffu, any = 0;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) fx_range_of(o[c], m, lowest, any);
+        __syncthreads();
+        info[threadIdx.x] = make_int4(int(m), int(lowest), int(any), 0);
+        __syncthreads();
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            const int4 q = info[32 * v + lane];
+            m = max(m, unsigned(q.x));
+            lowest = min(lowest, unsigned(q.y));
+            any |= unsigned(q.z);
+        }
+        if (site < vh && !slow) {
+            const FxSite f(m, lowest, any);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) f.store(A.out, i, 3 * w + c, o[c]);
+            if (w == 0) f.store_word(A.out, vh, i);
+        }
+    } else if (site < vh && !slow) {
+        double2 *q = static_cast<double2 *>(A.out);
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+            st_stream(PO == F64C ? q + size_t(i) * 12 + 3 * w + c : q + size_t(3 * w + c) * vh + i, make_double2(o[c].re, o[c].im));
+    }
+    if (slow && w == 0 && site < vh) fx_slow_site<PI, PX, PO, RECON, DAG, HASX>(A, i);
+}
+
+// Lattices up to this many sites per parity take the split hop: as many as
+// three of its CTAs per SM hold at once (3 x 152 x 32).  Measured, Q_tm whole
+// / split in us: 8^4 31 / 18, 8^3x16 31 / 20, 10^3x20 33 / 27, 12^3x24 37 /
+// 43, 16^4 41 / 59 (more warps, but each repeats the neighbour arithmetic and
+// the sums cross shared memory).
+#ifndef TM_FX_SPLIT_SITES
+#define TM_FX_SPLIT_SITES 14592
+#endif
+
+template <int PI, int PX, int PO, int RECON, bool DAG, bool HASX>
+static cudaError_t fx_launch(const FxArgs &A, cudaStream_t s)
+{
+    const unsigned vh = A.g.vh;
+    const bool signs = A.g.anti[1] || A.g.anti[2] || A.g.anti[3];
+    if (vh <= TM_FX_SPLIT_SITES) {
+        auto kern = k_fx_hop_split<PI, PX, PO, RECON, DAG, HASX, true>;
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(fx_split_bytes<RECON>()));
+        if (e != cudaSuccess) return e;
+        kern<<<(vh + 31) / 32, FX_SPLIT, fx_split_bytes<RECON>(), s>>>(A);
+    } else {
+        auto kern = signs ? k_fx_hop<PI, PX, PO, RECON, DAG, HASX, true> : k_fx_hop<PI, PX, PO, RECON, DAG, HASX, false>;
+        kern<<<(vh + FX_BLOCK - 1) / FX_BLOCK, FX_BLOCK, 0, s>>>(A);
+    }
+    return cudaGetLastError();
+}
 
 template <int RECON>
 static cudaError_t launch_f64_fields(const tm_gauge *U, bool dag, int p, const void *in, void *out, const void *x, const Coef &k,
                           cudaStream_t s, const SiteMap &m)
 {
-    auto kern = dag ? (x ? k_fx_hop<F64, F64, F64, RECON, true, true, true> : k_fx_hop<F64, F64, F64, RECON, true, false, true>)
-                    : (x ? k_fx_hop<F64, F64, F64, RECON, false, true, true> : k_fx_hop<F64, F64, F64, RECON, false, false, true>);
-    kern<<<fx_grid(U->geom.vh), FX_BLOCK, 0, s>>>(
-        FxArgs{U->geom, m, k, p, static_cast<const FxEntry *>(U->fx), static_cast<const double2 *>(U->links), in, x, out});
-    return cudaGetLastError();
+    const FxArgs A{U->geom, m, k, p, static_cast<const FxEntry *>(U->fx), static_cast<const double2 *>(U->links), in, x, out};
+    if (dag) return x ? fx_launch<F64, F64, F64, RECON, true, true>(A, s) : fx_launch<F64, F64, F64, RECON, true, false>(A, s);
+    return x ? fx_launch<F64, F64, F64, RECON, false, true>(A, s) : fx_launch<F64, F64, F64, RECON, false, false>(A, s);
 }
 
 cudaError_t launch_fx_hop(const tm_gauge *U, bool dag, int out_parity, const void *in, void *out, const void *x,
@@ -129,19 +274,18 @@ template <int PI, int RECON>
 static cudaError_t fx_qtm(const tm_gauge *U, bool stage_b, const void *in, void *tmp, void *out, const Coef &k, cudaStream_t s)
 {
     const Geom &g = U->geom;
-    const FxEntry *f = static_cast<const FxEntry *>(U->fx);
-    const double2 *l = static_cast<const double2 *>(U->links);
-    void *even = static_cast<char *>(tmp) + align256(fx_field_bytes(g.vh));
-    const bool signs = g.anti[1] || g.anti[2] || g.anti[3];
-    if (!stage_b) {
-        auto kern = signs ? k_fx_hop<FXF, F64, FXF, RECON, false, false, true> : k_fx_hop<FXF, F64, FXF, RECON, false, false, false>;
-        k_fx_field<PI><<<(g.vh + 127) / 128, 128, 0, s>>>(g.vh, in, even);
-        kern<<<fx_grid(g.vh), FX_BLOCK, 0, s>>>(FxArgs{g, U->map, k, 1, f, l, even, nullptr, tmp});
-    } else {
-        auto kern = signs ? k_fx_hop<FXF, PI, PI, RECON, false, true, true> : k_fx_hop<FXF, PI, PI, RECON, false, true, false>;
-        kern<<<fx_grid(g.vh), FX_BLOCK, 0, s>>>(FxArgs{g, U->map, k, 0, f, l, tmp, in, out});
+    FxArgs A{g, U->map, k, stage_b ? 0 : 1, static_cast<const FxEntry *>(U->fx), static_cast<const double2 *>(U->links), in, nullptr, tmp};
+    if (stage_b) {
+        A.in = tmp;
+        A.x = in;
+        A.out = out;
+        return fx_launch<FXF, PI, PI, RECON, false, true>(A, s);
     }
-    return cudaGetLastError();
+    if (g.vh <= TM_FX_SPLIT_SITES) return fx_launch<PI, F64, FXF, RECON, false, false>(A, s);
+    void *even = static_cast<char *>(tmp) + align256(fx_field_bytes(g.vh));
+    k_fx_field<PI><<<(g.vh + 127) / 128, 128, 0, s>>>(g.vh, in, even);
+    A.in = even;
+    return fx_launch<FXF, F64, FXF, RECON, false, false>(A, s);
 }
 
 cudaError_t launch_fx_qtm(const tm_gauge *U, bool canonical, bool stage_b, const void *in, void *tmp, void *out,

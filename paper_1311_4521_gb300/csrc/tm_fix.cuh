@@ -18,8 +18,8 @@
 // the ends of the exponent range, is computed with FP64 products instead
 // (fx_slow_site), and so is a gauge field with a link outside fx_link_ok.
 //
-// Measured (32^3x64, 18-real links): Q_tm 3.04 -> 0.80 ms, one hop 1.52 ->
-// 0.47 ms; 8^4: Q_tm 65 -> 31 us.  Launch B moves 4.9 TB/s, 0.73 of the
+// Measured (32^3x64, 18-real links): Q_tm 3.04 -> 0.77 ms, one hop 1.52 ->
+// 0.47 ms; 8^4, split over warps: Q_tm 65 -> 18 us.  Launch B moves 4.9 TB/s, 0.73 of the
 // measured copy bandwidth; its multiply-add pipe is busy 57 % of the time.
 // What it took beyond the integers (Q_tm at 32^3x64): multiply-adds from
 // plain C, not inline PTX 1.36 -> 1.02 ms; neighbours and links staged by
@@ -108,6 +108,44 @@ __device__ __forceinline__ const int *fx_words(const void *base, unsigned vh)
     return reinterpret_cast<const int *>(static_cast<const char *>(base) + size_t(FX_SPINOR_BLOCK) * fx_blocks(vh));
 }
 
+// Adds a component's high words without sign to a site's largest and lowest
+// (less one, so that zeros wrap and do not count), and all its bits but signs.
+__device__ __forceinline__ void fx_range_of(const cpx<double> &v, unsigned &m, unsigned &lowest, unsigned &bits)
+{
+    const unsigned p = unsigned(__double2hiint(v.re)) & 0x7fffffffu, q = unsigned(__double2hiint(v.im)) & 0x7fffffffu;
+    m = max(m, max(p, q));
+    lowest = min(lowest, min(p - 1u, q - 1u));
+    bits |= p | q | unsigned(__double2loint(v.re)) | unsigned(__double2loint(v.im));
+}
+
+// How a site is stored in a fixed-point field, from the range of its 12 components.
+struct FxSite {
+    bool raw;
+    int e;
+    unsigned span, from;
+    __device__ __forceinline__ FxSite(unsigned m, unsigned lowest, unsigned bits)
+    {
+        const bool zero = bits == 0;
+        const unsigned f = m >> 20;
+        span = zero ? 0u : f - ((lowest + 1u) >> 20);
+        raw = !zero && (f < FX_FMIN || f > FX_FMAX || span > unsigned(FX_SPAN));
+        e = zero ? FX_ZERO_E : int(f) - 1022;
+        from = zero ? 8000u : f + 4u;
+    }
+    __device__ __forceinline__ void store(void *base, unsigned i, int c, const cpx<double> &v) const
+    {
+        int4 o;
+        fx_split(v.re, from, 0u, o.x, o.y);
+        fx_split(v.im, from, 0u, o.z, o.w);
+        if (raw) o = make_int4(__double2hiint(v.re), __double2loint(v.re), __double2hiint(v.im), __double2loint(v.im));
+        st_stream(fx_entry(static_cast<int4 *>(base), FX_SPINOR_BLOCK, i) + 32 * c, o);
+    }
+    __device__ __forceinline__ void store_word(void *base, unsigned vh, unsigned i) const
+    {
+        st_stream(const_cast<int *>(fx_words(base, vh)) + i, raw ? FX_RAW : int(span << 16) | (e & 0xffff));
+    }
+};
+
 // Fixed-point fields read and written as FP64 sites.
 template <> struct SpinorIO<FXF> {
     using R = double;
@@ -130,33 +168,13 @@ template <> struct SpinorIO<FXF> {
     __device__ static void load(const void *base, unsigned vh, unsigned i, Spinor<R> &s) { load_raw(base, vh, i, s); }
     __device__ __forceinline__ static void store(void *base, unsigned vh, unsigned i, const Spinor<R> &s)
     {
-        int4 *b = fx_entry(static_cast<int4 *>(base), FX_SPINOR_BLOCK, i);
-        unsigned m = 0, lowest = 0xffffffffu;   // of the high words without sign; zeros wrap and do not count
-        unsigned bits = 0;
+        unsigned m = 0, lowest = 0xffffffffu, bits = 0;
 #pragma unroll
-        for (int c = 0; c < 12; ++c) {
-            const cpx<R> v = s[c / 3][c % 3];
-            const unsigned p = unsigned(__double2hiint(v.re)) & 0x7fffffffu, q = unsigned(__double2hiint(v.im)) & 0x7fffffffu;
-            m = max(m, max(p, q));
-            lowest = min(lowest, min(p - 1u, q - 1u));
-            bits |= p | q | unsigned(__double2loint(v.re)) | unsigned(__double2loint(v.im));
-        }
-        const bool zero = bits == 0;
-        const unsigned f = m >> 20;
-        const unsigned span = zero ? 0u : f - ((lowest + 1u) >> 20);
-        const bool raw = !zero && (f < FX_FMIN || f > FX_FMAX || span > unsigned(FX_SPAN));
-        const int e = zero ? FX_ZERO_E : int(f) - 1022;
-        const unsigned from = zero ? 8000u : f + 4u;
+        for (int c = 0; c < 12; ++c) fx_range_of(s[c / 3][c % 3], m, lowest, bits);
+        const FxSite f(m, lowest, bits);
 #pragma unroll
-        for (int c = 0; c < 12; ++c) {
-            const cpx<R> v = s[c / 3][c % 3];
-            int4 o;
-            fx_split(v.re, from, 0u, o.x, o.y);
-            fx_split(v.im, from, 0u, o.z, o.w);
-            if (raw) o = make_int4(__double2hiint(v.re), __double2loint(v.re), __double2hiint(v.im), __double2loint(v.im));
-            st_stream(b + 32 * c, o);
-        }
-        st_stream(const_cast<int *>(fx_words(base, vh)) + i, raw ? FX_RAW : int(span << 16) | (e & 0xffff));
+        for (int c = 0; c < 12; ++c) f.store(base, i, c, s[c / 3][c % 3]);
+        f.store_word(base, vh, i);
     }
 };
 
@@ -265,10 +283,10 @@ __device__ __forceinline__ bool fx_link_ok(const FxEntry (&u)[9])
 // words are read into registers (projected) before the next hop's copies
 // start, so they need one slot; the links need two.
 constexpr int FX_BLOCK = 64;   // threads per CTA of the fixed-point hops
-template <int RECON> struct FxStage {
-    static constexpr int NL = RECON / 2, WORDS = 12 + 2 * NL;
-    int4 *slot;   // this thread's first word; word w at slot[w * FX_BLOCK]
-    __device__ __forceinline__ int4 spinor(int c) const { return slot[c * FX_BLOCK]; }
+template <int RECON_, int BLOCK = FX_BLOCK> struct FxStage {
+    static constexpr int RECON = RECON_, NL = RECON / 2, WORDS = 12 + 2 * NL;
+    int4 *slot;   // this thread's first word; word w at slot[w * BLOCK]
+    __device__ __forceinline__ int4 spinor(int c) const { return slot[c * BLOCK]; }
     // the staged FP64 site
     __device__ __forceinline__ void site(Spinor<double> &s) const
     {
@@ -278,10 +296,10 @@ template <int RECON> struct FxStage {
             s[c / 3][c % 3] = {__hiloint2double(v.y, v.x), __hiloint2double(v.w, v.z)};
         }
     }
-    __device__ __forceinline__ int4 link(int q, int k) const { return slot[(12 + q * NL + k) * FX_BLOCK]; }
+    __device__ __forceinline__ int4 link(int q, int k) const { return slot[(12 + q * NL + k) * BLOCK]; }
     __device__ __forceinline__ void copy(int w, const void *src) const
     {
-        const unsigned dst = unsigned(__cvta_generic_to_shared(slot + w * FX_BLOCK));
+        const unsigned dst = unsigned(__cvta_generic_to_shared(slot + w * BLOCK));
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
     }
     // Starts the copies of one hop, the link into slot q: the words of the
@@ -311,8 +329,8 @@ template <int RECON> struct FxStage {
 //     re = K -+ ui (hr + hi),   im = K + ur (hi - hr).
 // Per sum the products with one low limb come first; shifted by a limb they
 // join the sum of the high ones.  Intermediate sums may wrap, results do not.
-template <int MU, int S, bool FWD, bool ALIGN, int RECON>
-__device__ __forceinline__ void fx_apply(const FxStage<RECON> &st, int q, const FxHalf &x, int d, FxSum &t)
+template <int MU, int S, bool FWD, bool ALIGN, class Stage>
+__device__ __forceinline__ void fx_apply(const Stage &st, int q, const FxHalf &x, int d, FxSum &t)
 {
     int sh[2][3], sl[2][3], dh[2][3], dl[2][3];   // -+(hr + hi) and hi - hr
 #pragma unroll
@@ -324,6 +342,7 @@ __device__ __forceinline__ void fx_apply(const FxStage<RECON> &st, int q, const 
             dh[s][c] = x.hi[s][c][1] - x.hi[s][c][0];
             dl[s][c] = x.lo[s][c][1] - x.lo[s][c][0];
         }
+    constexpr int RECON = Stage::RECON;
     FxEntry full[RECON == 12 ? 9 : 1];
     if constexpr (RECON == 12) {
 #pragma unroll
@@ -427,6 +446,12 @@ struct FxRange {
     unsigned fmax = 0, fmin = 0xffffffffu;   // high words met without sign; fmin less one, so that zeros do not count
     bool bad = false;
 };
+// Whether a site with these components is one that the integer path does not take.
+__device__ __forceinline__ bool fx_range_slow(const FxRange &r)
+{
+    const unsigned top = r.fmax >> 20, low = (r.fmin + 1u) >> 20;
+    return r.bad || top > FX_FMAX || (r.fmax && top - low > unsigned(FX_SPAN));
+}
 __device__ __forceinline__ void fx_from_half(const Half<double> &h, bool neg, FxHalf &x, FxSum &t, FxRange &q)
 {
     unsigned m = 0, lowest = 0xffffffffu;
@@ -472,8 +497,8 @@ __device__ __forceinline__ void fx_from_half(const Half<double> &h, bool neg, Fx
 
 // ---- the 8 hops
 // Starts the copies of hop K (2 mu, or 2 mu + 1 for the backward one).
-template <int P, int K, int RECON>
-__device__ __forceinline__ void fx_start(const Geom &g, const Nbrs &n, const FxLinks<RECON> &src, const void *in, const FxStage<RECON> &st)
+template <int P, int K, class Stage>
+__device__ __forceinline__ void fx_start(const Geom &g, const Nbrs &n, const FxLinks<Stage::RECON> &src, const void *in, const Stage &st)
 {
     constexpr int MU = K >> 1;
     const unsigned j = K & 1 ? n.bwd[MU] : n.fwd[MU];
@@ -484,11 +509,11 @@ __device__ __forceinline__ void fx_start(const Geom &g, const Nbrs &n, const FxL
     else st.start(K & 1, f + j, g.vh, u);
 }
 
-// Hop K and those after it.  SIGNS: whether directions other than time may
+// Hops K to LAST.  SIGNS: whether directions other than time may
 // have a boundary sign.
-template <int P, bool DAG, int K, bool SIGNS, int RECON>
-__device__ __forceinline__ void fx_hops(const Geom &g, const Nbrs &n, const FxLinks<RECON> &src, const void *in,
-                                        const FxStage<RECON> &st, const int4 *x0, size_t xstride, unsigned long long d,
+template <int P, bool DAG, int K, int LAST, bool SIGNS, class Stage>
+__device__ __forceinline__ void fx_hops(const Geom &g, const Nbrs &n, const FxLinks<Stage::RECON> &src, const void *in,
+                                        const Stage &st, const int4 *x0, size_t xstride, unsigned long long d,
                                         FxSum &t, FxRange &r)
 {
     st.wait();
@@ -507,10 +532,10 @@ __device__ __forceinline__ void fx_hops(const Geom &g, const Nbrs &n, const FxLi
         fx_from_half(h, neg, x, t, r);
     }
     __syncwarp();   // the site's words are read before the next copies start
-    if constexpr (K < 7) fx_start<P, K + 1>(g, n, src, in, st);
+    if constexpr (K < LAST) fx_start<P, K + 1>(g, n, src, in, st);
     else if (x0) st.start_site(x0, xstride);
-    fx_apply<MU, S, q == 0, P == FXF, RECON>(st, q, x, int(unsigned(d >> (8 * K)) & 0xffu), t);
-    if constexpr (K < 7) fx_hops<P, DAG, K + 1, SIGNS>(g, n, src, in, st, x0, xstride, d, t, r);
+    fx_apply<MU, S, q == 0, P == FXF>(st, q, x, int(unsigned(d >> (8 * K)) & 0xffu), t);
+    if constexpr (K < LAST) fx_hops<P, DAG, K + 1, LAST, SIGNS>(g, n, src, in, st, x0, xstride, d, t, r);
 }
 
 // Everything a fixed-point hop launch needs; a kernel parameter that device
@@ -542,6 +567,31 @@ __device__ __noinline__ void fx_slow_site(const FxArgs &A, unsigned i)
     SpinorIO<PO>::store(A.out, A.g.vh, i, o);
 }
 
+// The exponent of a site's sum, the largest of its 8 neighbours', and per hop
+// a byte of d: the shift that aligns it.  Returns whether the integer path
+// does not take the site.
+__device__ __forceinline__ bool fx_exponents(const Nbrs &n, const void *in, unsigned vh, int &sum_e, unsigned long long &d)
+{
+    const int *word = fx_words(in, vh);
+    int e[8], low = 0x7fff;
+    bool slow = false;
+    sum_e = FX_ZERO_E;
+#pragma unroll
+    for (int m = 0; m < 8; ++m) e[m] = ld_keep(word + (m & 1 ? n.bwd[m >> 1] : n.fwd[m >> 1]));
+#pragma unroll
+    for (int m = 0; m < 8; ++m) {
+        slow = slow || e[m] == FX_RAW;
+        const int span = e[m] >> 16;
+        e[m] = int(short(e[m] & 0xffff));
+        sum_e = max(sum_e, e[m]);
+        low = min(low, e[m] == FX_ZERO_E ? 0x7fff : e[m] - span);
+    }
+    d = 0;
+#pragma unroll
+    for (int m = 0; m < 8; ++m) d |= (unsigned long long)(unsigned(min(sum_e - e[m], 63))) << (8 * m);
+    return slow || sum_e - low > FX_SPAN;
+}
+
 // The hop at output site i; every thread of the warp calls it.  Returns
 // whether the site is one that the integer path does not take (acc is not
 // its hop then).  With x0 set, the 12 words at x0, xstride apart, are in the
@@ -562,31 +612,14 @@ __device__ __forceinline__ bool fx_hop_site(const FxArgs &A, unsigned i, const F
 #pragma unroll
         for (int c = 0; c < 3; ++c) t.re[s][c] = t.im[s][c] = 0;
     FxRange r;
-    unsigned long long d = 0;   // per hop a byte: the shift that aligns it to the site's exponent
+    unsigned long long d = 0;
     t.e = P == FXF ? FX_ZERO_E : -5000;
     bool slow = false;
     if constexpr (P == FXF) {
-        const int *word = fx_words(in, g.vh);
-        int e[8], low = 0x7fff;
-#pragma unroll
-        for (int m = 0; m < 8; ++m) e[m] = ld_keep(word + (m & 1 ? n.bwd[m >> 1] : n.fwd[m >> 1]));
-#pragma unroll
-        for (int m = 0; m < 8; ++m) {
-            slow = slow || e[m] == FX_RAW;
-            const int span = e[m] >> 16;
-            e[m] = int(short(e[m] & 0xffff));
-            t.e = max(t.e, e[m]);
-            low = min(low, e[m] == FX_ZERO_E ? 0x7fff : e[m] - span);
-        }
-        slow = slow || t.e - low > FX_SPAN;
-#pragma unroll
-        for (int m = 0; m < 8; ++m) d |= (unsigned long long)(unsigned(min(t.e - e[m], 63))) << (8 * m);
+        slow = fx_exponents(n, in, g.vh, t.e, d);
     }
-    fx_hops<P, DAG, 0, SIGNS>(g, n, src, in, st, x0, xstride, d, t, r);
-    if constexpr (P != FXF) {
-        const unsigned top = r.fmax >> 20, low = (r.fmin + 1u) >> 20;
-        slow = r.bad || top > FX_FMAX || (r.fmax && top - low > unsigned(FX_SPAN));
-    }
+    fx_hops<P, DAG, 0, 7, SIGNS>(g, n, src, in, st, x0, xstride, d, t, r);
+    if constexpr (P != FXF) slow = fx_range_slow(r);
     if (slow) return true;
     constexpr int bits = P == FXF ? FX_FIELD : FX_HALF;
 #pragma unroll

@@ -87,10 +87,13 @@ def has_fixed_links(g):
     return g.nbytes > 8 * g.vh * g.reconstruct * 8
 
 
-@pytest.mark.parametrize("dims,bc", [((4, 4, 4, 4), (-1, 1, 1, 1)), ((6, 4, 2, 10), (1, -1, -1, -1)),
-                                     ((10, 6, 2, 2), (-1, -1, 1, 1))])
-@pytest.mark.parametrize("recon", [18, 12])
-@pytest.mark.parametrize("kind", ["random", "near"])
+SMALL = [((4, 4, 4, 4), (-1, 1, 1, 1)), ((6, 4, 2, 10), (1, -1, -1, -1)), ((10, 6, 2, 2), (-1, -1, 1, 1))]
+# beyond the lattices whose hops are split over warps, ragged; with and without boundary signs in space
+LARGE = [((18, 10, 14, 12), (-1, 1, 1, 1), 18, "near"), ((14, 10, 18, 14), (1, 1, -1, 1), 12, "random")]
+
+
+@pytest.mark.parametrize("dims,bc,recon,kind",
+                         [(d, bc, r, k) for d, bc in SMALL for r in (18, 12) for k in ("random", "near")] + LARGE)
 def test_error_is_no_larger_than_with_fp64_products(ctx, dims, bc, recon, kind):
     U = F.gauge_field(dims, 911, kind)
     psi = F.gaussian_spinor(int(np.prod(dims)) // 2, 911, 1)
@@ -109,6 +112,8 @@ def test_error_is_no_larger_than_with_fp64_products(ctx, dims, bc, recon, kind):
 
 
 RANGES = ["1e200", "1e-200", "1e-290", "per_site", "per_component", "zero_sites", "point", "all_zero"]
+RANGE_CASES = [(r, (4, 6, 4, 8), k) for r in (18, 12) for k in RANGES] + [
+    (18, (18, 10, 14, 12), k) for k in ("1e-290", "per_component", "zero_sites")]
 
 
 def ranged(psi, kind):
@@ -130,12 +135,11 @@ def ranged(psi, kind):
     return psi * 0
 
 
-@pytest.mark.parametrize("kind", RANGES)
-@pytest.mark.parametrize("recon", [18, 12])
-def test_ranges(ctx, kind, recon):
+@pytest.mark.parametrize("recon,dims,kind", RANGE_CASES)
+def test_ranges(ctx, recon, dims, kind):
     """Every output component against extended precision, relative to the largest input components that enter it:
     8 roundings of the sums of 8 hops of magnitude at most 4 each."""
-    dims, bc = (4, 6, 4, 8), (-1, 1, 1, 1)
+    bc = (-1, 1, 1, 1)
     U = F.gauge_field(dims, 912, "random")
     psi = ranged(F.gaussian_spinor(int(np.prod(dims)) // 2, 912, 1), kind)
     E = Extended(dims, U, bc)
@@ -153,8 +157,8 @@ def test_ranges(ctx, kind, recon):
 
 
 @pytest.mark.parametrize("bad", [np.nan, np.inf, -np.inf, 1e305])
-def test_values_that_are_not_finite_spread_as_with_fp64_products(ctx, bad):
-    dims = (8, 4, 4, 8)
+@pytest.mark.parametrize("dims", [(8, 4, 4, 8), (18, 10, 14, 12)])
+def test_values_that_are_not_finite_spread_as_with_fp64_products(ctx, bad, dims):
     U = F.gauge_field(dims, 913, "random")
     psi = F.gaussian_spinor(int(np.prod(dims)) // 2, 913, 1)
     psi[17, 2, 1] = bad
@@ -193,7 +197,8 @@ def test_links_far_from_su3_use_fp64_products(ctx, change):
         g.close()
 
 
-@pytest.mark.parametrize("dims,names", [((16, 4, 4, 6), ["linear32", "linear96", "box8x2x2x1", "box4x4x4x2"])])
+@pytest.mark.parametrize("dims,names", [((16, 4, 4, 6), ["linear32", "linear96", "box8x2x2x1", "box8x4x4x1"]),
+                                        ((16, 8, 16, 16), ["linear32", "linear96", "box8x2x2x1", "box4x4x4x2"])])
 def test_maps_give_identical_bits(ctx, dims, names):
     from paper_1311_4521_gb300 import tmhop
     U = F.gauge_field(dims, 915, "near", 0.3)
