@@ -960,17 +960,18 @@ TM_HD void hop_dir_pair(const Geom &g, const Nbrs &n, const Src &src, const void
 // on "no instruction"); two hops per iteration were measured 2 % faster
 // than one, four slower.  Each link multiply is instantiated once; the
 // direction-dependent spin algebra is selected by small switches, and all
-// register arrays keep static indices.
+// register arrays keep static indices.  Does the hops k0 to k1 - 1 (2 mu
+// forward, 2 mu + 1 backward).
 template <int P, bool DAG, class Src>
 TM_HD void hop_site_rolled(const Geom &g, const Nbrs &n, const Src &src, const void *in,
-                           Spinor<typename SpinorIO<P>::R> &acc)
+                           Spinor<typename SpinorIO<P>::R> &acc, int k0 = 0, int k1 = 8)
 {
     using R = typename SpinorIO<P>::R;
     constexpr int SF = DAG ? +1 : -1;
     constexpr int SB = -SF;
     constexpr int kUnroll = TM_F64X_UNROLL;
 #pragma unroll kUnroll
-    for (int k = 0; k < 8; ++k) {
+    for (int k = k0; k < k1; ++k) {
         const int mu = k >> 1;
         const bool fwd = (k & 1) == 0;
         unsigned j;

@@ -137,11 +137,82 @@ cudaError_t launch_qtm(const tm_gauge *U, bool canonical, bool stage_b, const vo
     return qtm_canonical<12>(stage_b, g, U->map, U->links, in, tmp, out, k, s);
 }
 
+// The double-float hop with the 8 hops of a site dealt out to four warps, one
+// direction each, for lattices whose sites do not fill the GPU: a CTA covers
+// 32 sites.  A thread's 8 hops are a chain of some 27 us however few sites
+// there are.  The warps' partial sums meet in shared memory, are added in the
+// order of the directions, and warp w finishes spin w.  The site map is not
+// used (results do not depend on it).
+template <int RECON, bool DAG, bool HASX>
+__global__ void __launch_bounds__(128, TM_HOP_MINB(F64X))
+    k_hop_split(Geom g, int p, const typename LinkIO<F64X, RECON>::V *__restrict__ links, const void *__restrict__ in,
+                void *__restrict__ out, const void *__restrict__ x, Coef k)
+{
+    __shared__ float4 part[12][128];   // [component][direction, site]
+    const unsigned lane = threadIdx.x & 31, w = threadIdx.x >> 5, site = blockIdx.x * 32 + lane, i = min(site, g.vh - 1);
+    float4 xv[3];   // spin w of the re-read input
+    if (HASX)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) xv[c] = ld_keep(static_cast<const float4 *>(x) + size_t(3 * w + c) * g.vh + i);
+    {
+        Nbrs n;
+        neighbours(g, p, i, n);
+        const GlobalLinks<F64X, RECON> src{links, g.vh, i, p};
+        Spinor<dd> acc;
+#pragma unroll
+        for (int c = 0; c < 12; ++c) acc[c / 3][c % 3] = {dd(0.f), dd(0.f)};
+        // one loop for all warps: four copies of it, one per direction, overflowed the
+        // instruction cache (12^3x24, Q_tm: 86 us against 53)
+        hop_site_rolled<F64X, DAG>(g, n, src, in, acc, int(2 * w), int(2 * w + 2));
+#pragma unroll
+        for (int c = 0; c < 12; ++c) {
+            const cpx<dd> a = acc[c / 3][c % 3];
+            part[c][threadIdx.x] = make_float4(a.re.hi, a.re.lo, a.im.hi, a.im.lo);
+        }
+    }
+    __syncthreads();
+    if (site >= g.vh) return;
+    const dd z(0.f);
+    const int h = w < 2 ? 0 : 2;
+    const cpx<dd> a = {k.get(h, z), k.get(h + 1, z)}, b = {k.get(h + 4, z), k.get(h + 5, z)};
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        cpx<dd> hop = {z, z};
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            const float4 q = part[3 * w + c][32 * v + lane];
+            hop = hop + cpx<dd>{dd{q.x, q.y}, dd{q.z, q.w}};
+        }
+        cpx<dd> o = k.unit ? (w < 2 ? hop : -hop) : a * hop;
+        if (HASX) o = cmadd(b, cpx<dd>{dd{xv[c].x, xv[c].y}, dd{xv[c].z, xv[c].w}}, o);
+        st_stream(static_cast<float4 *>(out) + size_t(3 * w + c) * g.vh + i, make_float4(o.re.hi, o.re.lo, o.im.hi, o.im.lo));
+    }
+}
+
+// Lattices up to this many sites per parity take it.  Measured, Q_tm and the
+// result's unpacking, whole / split in us, 18-real links: 8^4 61 / 33, 12^3x24
+// 68 / 53, 14^3x28 72 / 72, 16^3x32 133 / 107, 20^3x40 252 / 241; 12-real,
+// whose warps each rebuild the rows they need: 10^3x20 75 / 46, 12^3x24 82 /
+// 82, 16^4 86 / 114.
+constexpr unsigned f64x_split_sites(int recon) { return recon == 18 ? 160000 : 16000; }
+
+template <int RECON>
+static cudaError_t hop_split(const Geom &g, bool dag, int p, const void *links, const void *in, void *out, const void *x,
+                             const Coef &k, cudaStream_t s)
+{
+    auto kern = dag ? (x ? k_hop_split<RECON, true, true> : k_hop_split<RECON, true, false>)
+                    : (x ? k_hop_split<RECON, false, true> : k_hop_split<RECON, false, false>);
+    kern<<<(g.vh + 31) / 32, 128, 0, s>>>(g, p, static_cast<const typename LinkIO<F64X, RECON>::V *>(links), in, out, x, k);
+    return cudaGetLastError();
+}
+
 template <int P, int RECON>
 static cudaError_t hop_dispatch(const Geom &g, bool dag, int p, const void *links, const void *in, void *out,
                                 const void *x, const Coef &k, cudaStream_t s, const SiteMap &m)
 {
     using V = typename LinkIO<P, RECON>::V;
+    if constexpr (P == F64X)
+        if (g.vh <= f64x_split_sites(RECON)) return hop_split<RECON>(g, dag, p, links, in, out, x, k, s);
     const V *l = static_cast<const V *>(links);
     const unsigned grid = map_grid(g, m);
     auto kern = dag ? (x ? k_hop<P, RECON, true, true> : k_hop<P, RECON, true, false>)
