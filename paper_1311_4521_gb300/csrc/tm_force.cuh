@@ -225,29 +225,45 @@ TM_HD void force_part_bwd(const Link<R> &u, const Spinor<R> &Rx, const Spinor<R>
 template <typename R> TM_HD void store_mat(double *o, const Mat<R> &m)
 {
 #pragma unroll
-    for (int a = 0; a < 3; ++a)
+    for (int k = 0; k < 9; ++k)
+        st_stream(reinterpret_cast<double2 *>(o) + k, make_double2(widen(m[k / 3][k % 3].re), widen(m[k / 3][k % 3].im)));
+}
+
+// A warp's 3x3 complex matrices, one per lane, to the 144-byte slots `slot` of
+// an FP64 force field (lanes with `on`): through the warp's 32 x 9 16-byte
+// words of shared memory, so that consecutive lanes write consecutive words
+// (evict-first, the field is written once); a lane writing its own matrix
+// touched 32 half sectors with every store.  Every lane of the warp calls it.
+template <typename R> __device__ __forceinline__ void store_mats(double *F, size_t slot, bool on, const Mat<R> &m, double2 *stage)
+{
+    const unsigned lane = threadIdx.x & 31;
 #pragma unroll
-        for (int b = 0; b < 3; ++b) {
-            const double2 v = make_double2(double(m[a][b].re), double(m[a][b].im));
-            st_stream(reinterpret_cast<double2 *>(o) + 3 * a + b, v);
-        }
+    for (int k = 0; k < 9; ++k) stage[9 * lane + k] = make_double2(widen(m[k / 3][k % 3].re), widen(m[k / 3][k % 3].im));
+    const unsigned mask = __ballot_sync(0xffffffffu, on);
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        const unsigned q = 32 * k + lane, from = q / 9;
+        const unsigned long long to = __shfl_sync(0xffffffffu, (unsigned long long)slot, int(from));
+        if ((mask >> from) & 1u) st_stream(reinterpret_cast<double2 *>(F) + to * 9 + (q - 9 * from), stage[q]);
+    }
+    __syncwarp();   // the words are read before the caller's next matrices
 }
 
 // Lexicographic index of the site with even-odd index i and parity p.
 TM_HD unsigned lex_of(const Geom &g, int p, unsigned i)
 {
-    unsigned r = i / g.hx;
-    unsigned y = r % g.ly;
-    r /= g.ly;
-    unsigned z = r % g.lz, t = r / g.lz;
+    const unsigned r = g.dhx.div(i), q = g.dly.div(r), y = r - q * unsigned(g.ly);
+    const unsigned t = g.dlz.div(q), z = q - t * unsigned(g.lz);
     return 2 * i + ((y + z + t + p) & 1);
 }
 
 // The force of link (mu, x) for x = (p, i).  Even sites hold X and Y (L =
-// gamma5 Y), odd sites Z and B.  Writes the 3x3 result to F[mu][lex(x)].
+// gamma5 Y), odd sites Z and B.
 template <int P, int RECON, int MU>
 TM_HD void force_site(const Geom &g, int p, unsigned i, const typename LinkIO<P, RECON>::V *links, const void *Xe,
-                      const void *Ye, const void *Zo, const void *Bo, double kappa2, int mode, double *F)
+                      const void *Ye, const void *Zo, const void *Bo, double kappa2, int mode,
+                      Mat<typename SpinorIO<P>::R> &m)
 {
     using R = typename SpinorIO<P>::R;
     using L = LinkIO<P, RECON>;
@@ -271,9 +287,7 @@ TM_HD void force_site(const Geom &g, int p, unsigned i, const typename LinkIO<P,
     }
     Link<R> u;
     L::load(links + size_t(4 * p + MU) * L::NCHUNK * g.vh, g.vh, i, u);
-    Mat<R> m;
     force_link<MU>(u, Rx, Lx, Rxp, Lxp, to_R<R>(kappa2), sgn, mode, m);
-    store_mat(F + (size_t(MU) * 2 * g.vh + lex_of(g, p, i)) * 18, m);
 }
 
 }  // namespace twm
