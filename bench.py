@@ -322,7 +322,14 @@ def gpu_arm(args) -> None:
     kb_gbs = vh * ab["kernel_b"] / (kb_ms * 1e-3) / 1e9
     traffic = args.traffic if args.traffic is not None else traffic_per_launch(prec, recon, vh)
     kname = f"k_hop<{prec.upper()},{recon},HASX> (Q_tm second launch: H_eo + gamma5 twisted update)"
-    if prec == "f64":
+    fixed = prec == "f64" and tmhop.tm_gauge_bytes(g.handle) > 8 * vh * 8 * recon   # links also in fixed point
+    if fixed:   # link products on the integer units: bound by memory and those, no longer by the FP64 pipe
+        kname = f"k_fx_hop<F64,{recon},HASX> (Q_tm second launch: H_eo + gamma5 twisted update)"
+        roofline = {"bound": "hbm", "achieved": round(kb_gbs, 1), "peak": hbm_peak, "unit": "GB/s",
+                    "frac": round(kb_gbs / hbm_peak, 4), "traffic": args.traffic, "kernel": kname,
+                    "peak_source": f"{hbm_src} HBM copy bandwidth", "tflops": round(kb_tflops, 4),
+                    "fp64_pipe_peak_tflops": round(fp64_peak, 4)}
+    elif prec == "f64":
         roofline = {"bound": "alu", "achieved": round(kb_tflops, 4), "peak": round(fp64_peak, 4),
                     "unit": "TFLOP/s", "frac": round(kb_tflops / fp64_peak, 4), "traffic": traffic,
                     "kernel": kname,
@@ -382,12 +389,12 @@ def gpu_arm(args) -> None:
         e2e = {"value": round(world * vh * ab["qtm"] / (e2e_ms * 1e-3) / 1e9, 2), "unit": "GB/s",
                "h2d_bytes_per_step": nbytes, "d2h_bytes_per_step": nbytes, "ms_per_step": round(e2e_ms, 4),
                "steps": ne,
-               # FP64: the two hops read and write the canonical host layout themselves; other formats add
-               # a pack and an unpack launch per field
-               "gpu_launches_per_step": 2 if prec == "f64" else 4,
+               # FP64: the input's conversion and the two hops read and write the canonical host layout
+               # themselves; other formats add a pack and an unpack launch per field
+               "gpu_launches_per_step": 3 if fixed else 2 if prec == "f64" else 4,
                "api": "tm_Qtm_host (pinned host fields, pipelined copies)"}
         del host_in, host_out
-    links_gb = tmhop.tm_gauge_bytes(g.handle) / 1e9
+    links_gb = tmhop.tm_gauge_bytes(g.handle) / (2 if fixed else 1) / 1e9   # the copy that the hops read
     g.close()
 
     # ---- storage-precision table (HBM-bound variants)
@@ -482,7 +489,7 @@ def gpu_arm(args) -> None:
                               f"+ {tmhop.tm_spinor_bytes(vh, tmhop.PREC[prec]) / 1e9:.3f} GB spinor read per step), no flush"),
             "gflops": round(gflops, 2), "roofline": roofline, "fp64_probe": probe, "hbm_peak_gbs": hbm_peak,
             "hbm_peak_source": hbm_src,
-            "e2e": e2e, "gpu_launches": 2 * args.steps, "clocks": ck, "precisions": table, "nd_doublet": nd, "clover": sw, "slabs": slabs, "f64x_equivalent": f64x, "cg": cg, "batch": batch, "grad": grad,
+            "e2e": e2e, "gpu_launches": (3 if fixed else 2) * args.steps, "clocks": ck, "precisions": table, "nd_doublet": nd, "clover": sw, "slabs": slabs, "f64x_equivalent": f64x, "cg": cg, "batch": batch, "grad": grad,
             "cpu_baseline": cpu, "paper_context": PAPER_CONTEXT,
         }
         print(json.dumps(line), flush=True)

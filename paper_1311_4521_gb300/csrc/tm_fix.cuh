@@ -440,8 +440,7 @@ __device__ __forceinline__ void fx_negate(FxHalf &x, int sg)
 }
 
 // ---- input in FP64
-// h (times -1 if neg) as limbs of 58 bits under the sum's exponent, which is
-// raised (to one more than h needs) where h does not fit.
+// The range of the components that a site's sum has met.
 struct FxRange {
     unsigned fmax = 0, fmin = 0xffffffffu;   // high words met without sign; fmin less one, so that zeros do not count
     bool bad = false;
@@ -452,6 +451,8 @@ __device__ __forceinline__ bool fx_range_slow(const FxRange &r)
     const unsigned top = r.fmax >> 20, low = (r.fmin + 1u) >> 20;
     return r.bad || top > FX_FMAX || (r.fmax && top - low > unsigned(FX_SPAN));
 }
+// h (times -1 if neg) as limbs of 58 bits under the sum's exponent, which is
+// raised (to one more than h needs) where h does not fit.
 __device__ __forceinline__ void fx_from_half(const Half<double> &h, bool neg, FxHalf &x, FxSum &t, FxRange &q)
 {
     unsigned m = 0, lowest = 0xffffffffu;

@@ -83,8 +83,8 @@ __global__ void __launch_bounds__(128, TM_HOP_MINB(P)) k_hop(Geom g, int p, cons
     SpinorIO<P>::store(out, g.vh, i, o);
 }
 
-// The two Q_tm launches of tm_Qtm_host for FP64 handles, on the caller's
-// canonical layout: launch A (PI = F64C) gathers its input from it, launch B
+// The two Q_tm launches of tm_Qtm_host for FP64 handles without fixed-point
+// links, on the caller's canonical layout: launch A (PI = F64C) gathers its input from it, launch B
 // re-reads it as x (PX = F64C) and writes its result in it (PO = F64C); the
 // odd temporary between them stays component-major.  The per-site
 // arithmetic is the hop's, so results equal tm_Qtm's on packed fields.
