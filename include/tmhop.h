@@ -237,7 +237,9 @@ tm_status tm_hopping_eo(tm_ctx *ctx, const tm_gauge *U, void *out_dev, const voi
  * Two launches: tmp_o = (1 + i mut gamma5)^-1 H_oe in_e into a scratch odd
  * field owned by ctx, then the fused even update (TM_F64 with fixed-point
  * links, above 14592 sites per parity: a third one before them that converts
- * in_e into a second scratch field).  out_e and in_e must not
+ * in_e into a second scratch field; the fixed-point scratch is a buffer of
+ * its own, and a call that is captured before one outside a capture has made
+ * it, or that finds no memory for it, does without).  out_e and in_e must not
  * overlap. */
 tm_status tm_Qtm(tm_ctx *ctx, const tm_gauge *U, void *out_e_dev, const void *in_e_dev, double kappa, double mu,
                  int sign, void *stream);

@@ -66,6 +66,32 @@ tm_status tm_ctx_scratch(tm_ctx *ctx, size_t bytes, void **ptr)
     return TM_OK;
 }
 
+tm_status tm_qtm_scratch(tm_ctx *ctx, const tm_gauge *U, cudaStream_t s, void **tmp, bool *fx)
+{
+    const size_t bytes = U->fx ? fx_qtm_bytes(U->geom.vh) : 0;
+    if (ctx->fx_scratch_bytes < bytes) {
+        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+        const cudaError_t q = cudaStreamIsCapturing(s, &capture);
+        if (q != cudaSuccess) (void)cudaGetLastError();   // the default stream while another one captures
+        if (q == cudaSuccess && capture == cudaStreamCaptureStatusNone) {
+            if (ctx->fx_scratch) {
+                const cudaError_t e = cudaFree(ctx->fx_scratch);
+                ctx->fx_scratch = nullptr;
+                ctx->fx_scratch_bytes = 0;
+                if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaFree(fixed-point scratch)");
+            }
+            const cudaError_t e = cudaMalloc(&ctx->fx_scratch, bytes);
+            if (e == cudaSuccess) ctx->fx_scratch_bytes = bytes;
+            else if (e != cudaErrorMemoryAllocation) return cuda_fail(ctx, e, "cudaMalloc(fixed-point scratch)");
+            else (void)cudaGetLastError();   // not sticky
+        }
+    }
+    *fx = bytes != 0 && ctx->fx_scratch_bytes >= bytes;
+    if (!*fx) return tm_ctx_scratch(ctx, spinor_bytes(U->geom.vh, U->prec), tmp);
+    *tmp = ctx->fx_scratch;
+    return TM_OK;
+}
+
 tm_status tm_ctx_reduce_buffer(tm_ctx *ctx, size_t bytes, void **ptr)
 {
     if (ctx->red_bytes < bytes) {
@@ -173,6 +199,7 @@ void tm_ctx_destroy(tm_ctx *ctx)
 {
     if (!ctx) return;
     if (ctx->scratch) cudaFree(ctx->scratch);
+    if (ctx->fx_scratch) cudaFree(ctx->fx_scratch);
     if (ctx->ws) cudaFree(ctx->ws);
     if (ctx->stage) cudaFree(ctx->stage);
     if (ctx->bq) cudaFree(ctx->bq);
@@ -342,14 +369,15 @@ tm_status tm_Qtm(tm_ctx *ctx, const tm_gauge *U, void *out_e_dev, const void *in
     if (sign != 1 && sign != -1) return fail(ctx, TM_ERR_ARG, "tm_Qtm: sign must be +1 or -1");
     if (out_e_dev == in_e_dev) return fail(ctx, TM_ERR_ARG, "tm_Qtm: out and in must not overlap");
     void *tmp = nullptr;
-    tm_status st = tm_ctx_scratch(ctx, qtm_bytes(U), &tmp);
+    bool fx = false;
+    cudaStream_t s = (cudaStream_t)stream;
+    tm_status st = tm_qtm_scratch(ctx, U, s, &tmp, &fx);
     if (st != TM_OK) return st;
     double mut = 2.0 * kappa * mu * sign;
-    cudaStream_t s = (cudaStream_t)stream;
     tm_trace_mark(ctx, 0, s);
-    TM_CUDA(ctx, launch_qtm(U, false, false, in_e_dev, tmp, out_e_dev, coef_qtm_a_scaled(kappa, mut), s));
+    TM_CUDA(ctx, launch_qtm(U, fx, false, false, in_e_dev, tmp, out_e_dev, coef_qtm_a_scaled(kappa, mut), s));
     tm_trace_mark(ctx, 1, s);
-    TM_CUDA(ctx, launch_qtm(U, false, true, in_e_dev, tmp, out_e_dev, coef_qtm_b_unit(mut), s));
+    TM_CUDA(ctx, launch_qtm(U, fx, false, true, in_e_dev, tmp, out_e_dev, coef_qtm_b_unit(mut), s));
     tm_trace_mark(ctx, 2, s);
     return TM_OK;
 }

@@ -84,7 +84,8 @@ extern "C" tm_status tm_Qtm_host(tm_ctx *ctx, const tm_gauge *U, int n, double *
     tm_status st = grow_stage(ctx, 2 * (2 * cba + 2 * pba));
     if (st != TM_OK) return st;
     void *tmp = nullptr;  // tm_Qtm's scratch, grown now so that no call below reallocates it
-    st = tm_ctx_scratch(ctx, qtm_bytes(U), &tmp);
+    bool fx = false;
+    st = tm_qtm_scratch(ctx, U, (cudaStream_t)stream, &tmp, &fx);
     if (st != TM_OK) return st;
     char *base = static_cast<char *>(ctx->stage);
     double *can_in[2], *can_out[2];
@@ -122,9 +123,9 @@ extern "C" tm_status tm_Qtm_host(tm_ctx *ctx, const tm_gauge *U, int n, double *
             if (e == cudaSuccess) e = cudaStreamWaitEvent(s, ev.unpacked[q], 0);
             if (e == cudaSuccess) {
                 tm_trace_mark(ctx, 0, s);
-                e = launch_qtm(U, true, false, can_in[q], tmp, can_out[q], ka, s);
+                e = launch_qtm(U, fx, true, false, can_in[q], tmp, can_out[q], ka, s);
                 tm_trace_mark(ctx, 1, s);
-                if (e == cudaSuccess) e = launch_qtm(U, true, true, can_in[q], tmp, can_out[q], kb, s);
+                if (e == cudaSuccess) e = launch_qtm(U, fx, true, true, can_in[q], tmp, can_out[q], kb, s);
                 tm_trace_mark(ctx, 2, s);
             }
             if (e == cudaSuccess) e = cudaEventRecord(ev.multiplied[q], s);

@@ -41,6 +41,8 @@ struct tm_ctx {
     std::string err;
     void *scratch = nullptr;       // odd-parity temporaries of Q_tm and friends
     size_t scratch_bytes = 0;
+    void *fx_scratch = nullptr;    // fixed-point temporaries of Q_tm (tm_qtm_scratch)
+    size_t fx_scratch_bytes = 0;
     int sm_count = 0;
     std::vector<cudaEvent_t> trace;  // events recorded at kernel boundaries (tm_ctx_trace)
     void *ws = nullptr;              // solver workspace (grow-only)
@@ -112,6 +114,12 @@ inline double reliable_delta_for(double delta, int inner_prec)
 
 // Grows the context's scratch buffer to at least `bytes` and returns it.
 tm_status tm_ctx_scratch(tm_ctx *ctx, size_t bytes, void **ptr);
+// The odd temporary of Q_tm on stream s for launch_qtm: fixed-point fields
+// (*fx) for handles with fixed-point links, in a buffer of their own, so that
+// a graph captured around another operator keeps the scratch that it was
+// captured with; where that buffer would have to grow while a stream
+// captures, or does not fit the device, a field in the handle's precision.
+tm_status tm_qtm_scratch(tm_ctx *ctx, const tm_gauge *U, cudaStream_t s, void **tmp, bool *fx);
 // Grows the context's solver workspace to at least `bytes` and returns it.
 tm_status tm_ctx_workspace(tm_ctx *ctx, size_t bytes, void **ptr);
 // Grows the context's reduction buffer (partials of tm_spinor_dot) and returns it.
@@ -163,11 +171,10 @@ cudaError_t launch_fx_qtm(const tm_gauge *U, bool canonical, bool stage_b, const
 // Fills the geometry of a lattice; returns false if the extents are invalid.
 bool make_geom(const int dims[4], const int bc[4], Geom &g);
 
-// The two stages of Q_tm and their odd temporary (the scratch of qtm_bytes):
-// stage A in -> tmp, stage B tmp -> out with in re-read.  canonical: FP64
-// fields in the caller's canonical layout.
-size_t qtm_bytes(const tm_gauge *U);
-cudaError_t launch_qtm(const tm_gauge *U, bool canonical, bool stage_b, const void *in, void *tmp, void *out,
+// The two stages of Q_tm, tmp and fx from tm_qtm_scratch: stage A in -> tmp,
+// stage B tmp -> out with in re-read.  canonical: FP64 fields in the caller's
+// canonical layout.
+cudaError_t launch_qtm(const tm_gauge *U, bool fx, bool canonical, bool stage_b, const void *in, void *tmp, void *out,
                        const Coef &k, cudaStream_t s);
 
 // Launchers (tm_kernels.cu).  All enqueue on `s` and return the launch status.

@@ -122,14 +122,12 @@ static cudaError_t qtm_canonical(bool stage_b, const Geom &g, const SiteMap &m, 
     return cudaGetLastError();
 }
 
-size_t qtm_bytes(const tm_gauge *U) { return U->fx ? fx_qtm_bytes(U->geom.vh) : spinor_bytes(U->geom.vh, U->prec); }
-
-cudaError_t launch_qtm(const tm_gauge *U, bool canonical, bool stage_b, const void *in, void *tmp, void *out,
+cudaError_t launch_qtm(const tm_gauge *U, bool fx, bool canonical, bool stage_b, const void *in, void *tmp, void *out,
                        const Coef &k, cudaStream_t s)
 {
     const Geom &g = U->geom;
     if (g.vh == 0) return cudaSuccess;
-    if (U->fx) return launch_fx_qtm(U, canonical, stage_b, in, tmp, out, k, s);
+    if (fx) return launch_fx_qtm(U, canonical, stage_b, in, tmp, out, k, s);
     if (!canonical) {
         return stage_b ? launch_hop(U, false, TM_EO, tmp, out, in, k, s) : launch_hop(U, false, TM_OE, in, tmp, nullptr, k, s);
     }
