@@ -187,12 +187,18 @@ __global__ void __launch_bounds__(128, TM_HOP_MINB(F64X))
     }
 }
 
-// Lattices up to this many sites per parity take it.  Measured, Q_tm and the
-// result's unpacking, whole / split in us, 18-real links: 8^4 61 / 33, 12^3x24
-// 68 / 53, 14^3x28 72 / 72, 16^3x32 133 / 107, 20^3x40 252 / 241; 12-real,
+// Lattices that take it: up to 16000 sites per parity, and for 18-real links
+// from the second wave of the whole hop (more than 2 x 152 CTAs of 128) to
+// 160000.  Measured, Q_tm and the result's unpacking, whole / split in us,
+// 18-real links: 8^4 61 / 33, 16^3x32 133 / 107, 20^3x40 252 / 241; 12-real,
 // whose warps each rebuild the rows they need: 10^3x20 75 / 46, 12^3x24 82 /
-// 82, 16^4 86 / 114.
-constexpr unsigned f64x_split_sites(int recon) { return recon == 18 ? 160000 : 16000; }
+// 82, 16^4 86 / 114.  Between the two ranges the whole hop is one wave of 23
+// to 25 us: a hop 14^3x28 25.0 / 26.1; 12^3x24 with unpacking, one call
+// after another, 36.9 on every run against 30, 37 and 41.
+inline bool f64x_split(int recon, unsigned vh)
+{
+    return vh <= 16000 || (recon == 18 && vh > 2 * 152 * 128 && vh <= 160000);
+}
 
 template <int RECON>
 static cudaError_t hop_split(const Geom &g, bool dag, int p, const void *links, const void *in, void *out, const void *x,
@@ -210,7 +216,7 @@ static cudaError_t hop_dispatch(const Geom &g, bool dag, int p, const void *link
 {
     using V = typename LinkIO<P, RECON>::V;
     if constexpr (P == F64X)
-        if (g.vh <= f64x_split_sites(RECON)) return hop_split<RECON>(g, dag, p, links, in, out, x, k, s);
+        if (f64x_split(RECON, g.vh)) return hop_split<RECON>(g, dag, p, links, in, out, x, k, s);
     const V *l = static_cast<const V *>(links);
     const unsigned grid = map_grid(g, m);
     auto kern = dag ? (x ? k_hop<P, RECON, true, true> : k_hop<P, RECON, true, false>)
