@@ -29,6 +29,7 @@ __global__ void __launch_bounds__(FX_BLOCK, 6) k_cg_fx_hop(const __grid_constant
     const int4 *x0 = HASX && PX == F64 ? static_cast<const int4 *>(A.x) + i : nullptr;
     Spinor<double> acc, xs, o;
     const bool slow = fx_hop_site<PI, RECON, false, SIGNS>(A, i, st, x0, vh, acc);
+    if (HASX && PX == F64) st.wait();   // on every path: no thread leaves with copies to its slots under way
     double nrm = 0.0;
     if (site < vh) {
         if (slow) {   // stored, then read back (HOP_UPDATE: from a field that serves nothing else)
@@ -36,7 +37,6 @@ __global__ void __launch_bounds__(FX_BLOCK, 6) k_cg_fx_hop(const __grid_constant
             if (MODE != HOP_PLAIN) SpinorIO<PO>::load_raw(A.out, vh, i, o);
         } else {
             if (HASX && PX == F64) {
-                st.wait();
                 st.site(xs);
             } else if (HASX) {
                 SpinorIO<PX>::load_raw(A.x, vh, i, xs);

@@ -88,15 +88,13 @@ __global__ void __launch_bounds__(FX_BLOCK, TM_FX_MINB)
     const int4 *x0 = HASX ? static_cast<const int4 *>(A.x) + (PX == F64C ? size_t(i) * 12 : size_t(i)) : nullptr;
     Spinor<double> acc, xs, o;
     const bool slow = fx_hop_site<PI, RECON, DAG, SIGNS>(A, i, st, x0, PX == F64C ? 1 : g.vh, acc);
+    if (HASX) st.wait();   // on every path: no thread leaves with copies to its slots under way
     if (site >= g.vh) return;
     if (slow) {
         fx_slow_site<PI, PX, PO, RECON, DAG, HASX>(A, i);
         return;
     }
-    if (HASX) {
-        st.wait();
-        st.site(xs);
-    }
+    if (HASX) st.site(xs);
     epilogue(A.k, acc, HASX ? &xs : nullptr, o);
     SpinorIO<PO>::store(A.out, g.vh, i, o);
 }

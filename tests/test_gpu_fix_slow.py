@@ -1,0 +1,48 @@
+"""Sites that the fixed-point FP64 hop leaves to FP64 products (tm_fix.cuh),
+in CTAs that also hold threads past the lattice's end: the operator and the
+solver's hops against references, over boundary signs in space and both link
+formats."""
+import numpy as np
+import pytest
+
+import oracle as O
+from paper_1311_4521_gb300 import fields as F
+
+pytestmark = pytest.mark.gpu
+KAPPA, MU = 0.1394, 0.0015
+EPS = 2.0 ** -52
+# 15120 and 15840 sites per parity: beyond the split hop, with a partial last CTA of 64
+SIGNED = [((18, 10, 14, 12), (-1, 1, 1, 1), 18), ((22, 6, 10, 24), (1, -1, 1, -1), 12)]
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    from paper_1311_4521_gb300 import tmhop
+    c = tmhop.Context(0)
+    yield c
+    c.close()
+
+
+def rel(a, b):
+    return float(np.linalg.norm((a - b).ravel()) / np.linalg.norm(b.ravel()))
+
+
+def wide(vh, seed):
+    """A Gaussian field with components of every eighth site 2^-40 to 2^-30 of the others': their neighbours are
+    slow sites, one to all of a warp's."""
+    rng = np.random.default_rng(seed)
+    psi = F.gaussian_spinor(vh, seed, 1)
+    psi[::8] *= 2.0 ** -rng.integers(30, 41, size=psi[::8].shape)
+    return psi
+
+
+@pytest.mark.parametrize("dims,bc,recon", SIGNED)
+def test_slow_sites_next_to_threads_past_the_end(ctx, dims, bc, recon):
+    vh = int(np.prod(dims)) // 2
+    U, psi = F.gauge_field(dims, 961, "near", 0.3), wide(vh, 961)
+    g, src = ctx.gauge(dims, U, "f64", recon, bc), ctx.pack(psi, "f64")
+    outs = [ctx.Qtm(g, ctx.empty(vh, "f64"), src, KAPPA, MU) for _ in range(20)]
+    got = [ctx.unpack(o, vh, "f64").cpu().numpy() for o in outs]
+    assert rel(got[0], O.Qtm(dims, U, psi, KAPPA, MU, bc=bc)) < 8 * EPS   # the operator's error and the oracle's, each below EPS or a few
+    assert all(np.array_equal(got[0], v) for v in got)
+    g.close()
