@@ -19,6 +19,22 @@ struct CgFxArgs {
     int gate;
 };
 
+// Site i of a field that this thread has just stored.  Not through the
+// read-only path of SpinorIO's loads, which is for memory that nothing writes
+// during the kernel.
+template <int P> __device__ __forceinline__ void fx_read_back(const void *base, unsigned vh, unsigned i, Spinor<double> &s)
+{
+    const volatile int4 *b = P == FXF ? fx_entry(static_cast<const int4 *>(base), FX_SPINOR_BLOCK, i)
+                                      : static_cast<const int4 *>(base) + i;
+    const int word = P == FXF ? static_cast<const volatile int *>(fx_words(base, vh))[i] : FX_RAW;
+#pragma unroll
+    for (int c = 0; c < 12; ++c) {
+        const volatile int4 &q = b[c * (P == FXF ? size_t(32) : size_t(vh))];
+        const int4 v = make_int4(q.x, q.y, q.z, q.w);
+        s[c / 3][c % 3] = P == FXF ? fx_component(v, word) : cpx<double>{__hiloint2double(v.y, v.x), __hiloint2double(v.w, v.z)};
+    }
+}
+
 template <int PI, int PX, int PO, int RECON, int MODE, bool HASX, bool SIGNS>
 __global__ void __launch_bounds__(FX_BLOCK, 6) k_cg_fx_hop(const __grid_constant__ FxArgs A, const __grid_constant__ CgFxArgs C)
 {
@@ -34,7 +50,7 @@ __global__ void __launch_bounds__(FX_BLOCK, 6) k_cg_fx_hop(const __grid_constant
     if (site < vh) {
         if (slow) {   // stored, then read back (HOP_UPDATE: from a field that serves nothing else)
             fx_slow_site<PI, PX, PO, RECON, false, HASX>(A, i);
-            if (MODE != HOP_PLAIN) SpinorIO<PO>::load_raw(A.out, vh, i, o);
+            if (MODE != HOP_PLAIN) fx_read_back<PO>(A.out, vh, i, o);
         } else {
             if (HASX && PX == F64) {
                 st.site(xs);

@@ -146,6 +146,15 @@ struct FxSite {
     }
 };
 
+// A stored component of a site with word `word`, in FP64.
+__device__ __forceinline__ cpx<double> fx_component(const int4 &v, int word)
+{
+    if (word == FX_RAW) return {__hiloint2double(v.x, v.y), __hiloint2double(v.z, v.w)};
+    const int e = int(short(word & 0xffff));
+    return {fx_to_double(((long long)v.x << FX_LIMB) + v.y, e, FX_FIELD),
+            fx_to_double(((long long)v.z << FX_LIMB) + v.w, e, FX_FIELD)};
+}
+
 // Fixed-point fields read and written as FP64 sites.
 template <> struct SpinorIO<FXF> {
     using R = double;
@@ -153,16 +162,8 @@ template <> struct SpinorIO<FXF> {
     {
         const int4 *b = fx_entry(static_cast<const int4 *>(base), FX_SPINOR_BLOCK, i);
         const int word = fx_words(base, vh)[i];
-        const int e = int(short(word & 0xffff));
 #pragma unroll
-        for (int c = 0; c < 12; ++c) {
-            const int4 v = b[32 * c];
-            if (word == FX_RAW)
-                s[c / 3][c % 3] = {__hiloint2double(v.x, v.y), __hiloint2double(v.z, v.w)};
-            else
-                s[c / 3][c % 3] = {fx_to_double(((long long)v.x << FX_LIMB) + v.y, e, FX_FIELD),
-                                   fx_to_double(((long long)v.z << FX_LIMB) + v.w, e, FX_FIELD)};
-        }
+        for (int c = 0; c < 12; ++c) s[c / 3][c % 3] = fx_component(b[32 * c], word);
         return R(1);
     }
     __device__ static void load(const void *base, unsigned vh, unsigned i, Spinor<R> &s) { load_raw(base, vh, i, s); }

@@ -46,3 +46,29 @@ def test_slow_sites_next_to_threads_past_the_end(ctx, dims, bc, recon):
     assert rel(got[0], O.Qtm(dims, U, psi, KAPPA, MU, bc=bc)) < 8 * EPS   # the operator's error and the oracle's, each below EPS or a few
     assert all(np.array_equal(got[0], v) for v in got)
     g.close()
+
+
+@pytest.mark.parametrize("inner", ["f64", "f32"])
+@pytest.mark.parametrize("dims,bc,recon", SIGNED)
+def test_solve_with_a_source_of_wide_range(ctx, dims, bc, recon, inner):
+    """A point source: the first iterations meet slow sites in every hop.  FP64 CG takes the oracle's iterations
+    but for rounding; what a wrong hop or update costs is more of them, or a residual that does not follow."""
+    vh = int(np.prod(dims)) // 2
+    U = F.gauge_field(dims, 962, "near", 0.3)
+    b = np.zeros((vh, 4, 3), dtype=np.complex128)
+    b[vh // 3, 1, 2] = 1.0
+    b[vh // 2] = 2.0 ** -35 * (1 - 0.5j)
+    g = ctx.gauge(dims, U, "f64", recon, bc)
+    lo = None if inner == "f64" else ctx.gauge(dims, U, inner, 12, bc)
+    x = ctx.empty(vh, "f64").zero_()
+    st, info = ctx.cg(g, x, ctx.pack(b, "f64"), 0.12, 0.05, 1e-10, 1000, lo)
+    assert st == 0 and info["true_relres"] <= 1e-10
+    xs = ctx.unpack(x, vh, "f64").cpu().numpy()
+    back = O.Qtm(dims, U, O.Qtm(dims, U, xs, 0.12, 0.05, bc=bc), 0.12, -0.05, bc=bc)
+    assert rel(back, b) < 2e-10
+    if inner == "f64":
+        iters = O.cg_QdagQ(dims, U, b, 0.12, 0.05, 1e-10, 1000, bc=bc)[1]
+        assert abs(info["iters"] - iters) <= 1 + iters // 50
+    g.close()
+    if lo:
+        lo.close()
