@@ -545,10 +545,7 @@ extern "C" tm_status tm_cg_QdagQ(tm_ctx *ctx, const tm_gauge *U_hi, const tm_gau
         e = cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking);
         if (e == cudaSuccess) e = S.loop_graph(cap, &exec, handles);
         if (e == cudaSuccess) {
-            h.loop = handles[0];
-            h.update = handles[1];
-            h.segment = K;
-            h.loops = 0;
+            h.set_graph(handles[0], w.mixed, handles[1], K);
             e = cudaMemcpyAsync(w.s, &h, sizeof h, cudaMemcpyHostToDevice, s);
         }
         if (e != cudaSuccess) {

@@ -31,10 +31,23 @@ struct CgScalars {
     int mixed;       // 1: reduced-precision inner solver with reliable updates
     int nreliable;   // FP64 residual recomputations so far
     unsigned ticket; // last-block-done counter of the current reduction
-    // graph replay (zero without): the handles of the loop over iterations and
-    // of the reliable update inside it, iterations of the current segment
+    // graph replay: the handles of the loop over iterations and of the
+    // reliable update inside it (any value, zero too, may be a handle, so
+    // their presence has flags), iterations of the current segment
     unsigned long long loop, update;
+    int has_loop, has_update;
     int segment, loops;
+    // The next launches run under a graph with these handles (update: its
+    // conditional reliable update, if there is one) in segments of n iterations.
+    void set_graph(unsigned long long loop_handle, bool with_update, unsigned long long update_handle, int n)
+    {
+        loop = loop_handle;
+        update = update_handle;
+        has_loop = 1;
+        has_update = with_update ? 1 : 0;
+        segment = n;
+        loops = 0;
+    }
 };
 
 // Gates of the iteration kernels: 0 always run, 1 skip once the solve is
@@ -44,15 +57,19 @@ __device__ __forceinline__ bool gated(const CgScalars *s, int gate)
     return gate == 1 ? s->done != 0 : gate == 2 ? s->reliable == 0 : false;
 }
 
-// The end of an iteration: whether the graph's loop runs another one.  Every
-// path of an iteration's last kernel comes here, so a segment ends after at
-// most `segment` iterations.
-__device__ __forceinline__ void cg_loop_end(CgScalars *s)
+// The end of an iteration of the graph's loop: whether it runs another one.
+TM_HD bool cg_loop_more(CgScalars *s)
 {
-    if (!s->loop) return;
     const bool more = !s->done && ++s->loops < s->segment;
     if (!more) s->loops = 0;
-    cudaGraphSetConditional(s->loop, more);
+    return more;
+}
+
+// Every path of an iteration's last kernel comes here, so a segment ends
+// after at most `segment` iterations.
+__device__ __forceinline__ void cg_loop_end(CgScalars *s)
+{
+    if (s->has_loop) cudaGraphSetConditional(s->loop, cg_loop_more(s));
 }
 
 enum Fin { FIN_PAP, FIN_RR_UPDATE, FIN_RR_TRUE, FIN_RR_CHECK, FIN_BB, FIN_ROLL };
@@ -84,7 +101,7 @@ __device__ __forceinline__ void cg_finish(int op, double total, CgScalars *s)
         } else if (stop) {
             s->pending = 1;
         }
-        if (s->update) cudaGraphSetConditional(s->update, s->reliable != 0);
+        if (s->has_update) cudaGraphSetConditional(s->update, s->reliable != 0);
         break;
     }
     case FIN_RR_TRUE:
