@@ -441,9 +441,11 @@ tm_status tm_force_ex(tm_ctx *ctx, const tm_gauge *U, double *F_dev, const void 
  * tm_Qtm: the first call for a batch (its handles, field pointers, lattice
  * sizes and stream) uploads its tables and, for a new batch shape, times
  * launch configurations (which synchronises the stream); a repeated call
- * with the same batch only launches.  Batched calls on one ctx that overlap on
- * different streams are not supported (the ctx synchronises the previous
- * stream when the stream changes). */
+ * with the same batch only launches.  A capturing stream takes only such a
+ * repeated call; a batch that is new to ctx is refused (TM_ERR_CUDA).
+ * Batched calls on one ctx that overlap on different streams are not
+ * supported (the ctx synchronises the previous stream when the stream
+ * changes). */
 tm_status tm_Qtm_batch(tm_ctx *ctx, int nsys, const tm_gauge *const *U, void *const *out_e, const void *const *in_e,
                        double kappa, double mu, int sign, void *stream);
 

@@ -300,12 +300,11 @@ int zband_for(const Geom &g, unsigned ts)
 bool band_order(int prec) { return prec != F16; }
 
 // Fills a hop table for pass width nrb and uploads it to `dev` (capacity
-// ngroups).  The copy from pageable memory has taken the data when it returns.
-cudaError_t build_table(const std::vector<BGroup> &tmpl, int nrb, unsigned grid_cap, HopTable &t, BGroup *dev,
-                        cudaStream_t st, std::vector<BGroup> &host, const StageArgs &sa = StageArgs{},
-                        bool band = true)
+// ngroups).
+cudaError_t build_table(tm_ctx *ctx, const std::vector<BGroup> &tmpl, int nrb, unsigned grid_cap, HopTable &t,
+                        BGroup *dev, cudaStream_t st, const StageArgs &sa = StageArgs{}, bool band = true)
 {
-    host = tmpl;
+    std::vector<BGroup> host = tmpl;
     const int w = code_nrb(nrb), rpt = code_rpt(nrb);
     const unsigned ts = w > 1 ? BT / w : BT;
     unsigned item = 0;
@@ -327,7 +326,7 @@ cudaError_t build_table(const std::vector<BGroup> &tmpl, int nrb, unsigned grid_
     t.grid = std::max(1u, std::min(item, grid_cap));
     t.ngroups = int(host.size());
     t.dev = dev;
-    return cudaMemcpyAsync(dev, host.data(), sizeof(BGroup) * host.size(), cudaMemcpyHostToDevice, st);
+    return ctx->tables.upload(dev, host.data(), sizeof(BGroup) * host.size(), st);
 }
 
 // Times a candidate hop table with (parity 1, rin -> rout) launches; returns
@@ -375,12 +374,11 @@ cudaError_t tune_hop_table(tm_ctx *ctx, int prec, int recon, const std::vector<B
         key += "/" + std::to_string(g.g.vh) + "x" + std::to_string(g.nrhs);
     }
     const unsigned sms = unsigned(std::max(1, ctx->sm_count));
-    std::vector<BGroup> host;
     if (ctx->batch_code >= 0) {   // a configuration set by the caller, where this format has it
         const std::vector<int> ok = nrb_candidates(prec, recon, std::max(nrhs_max, 2), sa != nullptr);
         if (std::find(ok.begin(), ok.end(), ctx->batch_code) != ok.end()) {
             const unsigned dcap = ctx->batch_code == STAGE_CODE ? sms : 1u << 30;
-            return build_table(tmpl, ctx->batch_code, ctx->batch_cap ? ctx->batch_cap : dcap, out, dev, st, host, sta,
+            return build_table(ctx, tmpl, ctx->batch_code, ctx->batch_cap ? ctx->batch_cap : dcap, out, dev, st, sta,
                                band_order(prec));
         }
     }
@@ -405,7 +403,7 @@ cudaError_t tune_hop_table(tm_ctx *ctx, int prec, int recon, const std::vector<B
         }
     }
     if (it != ctx->tuned.end())
-        return build_table(tmpl, it->second.first, it->second.second, out, dev, st, host, sta, band_order(prec));
+        return build_table(ctx, tmpl, it->second.first, it->second.second, out, dev, st, sta, band_order(prec));
     float best = 1e30f;
     int best_nrb = 1;
     unsigned best_cap = 1u << 30;
@@ -414,7 +412,7 @@ cudaError_t tune_hop_table(tm_ctx *ctx, int prec, int recon, const std::vector<B
         for (unsigned cap : caps) {
             if (nrb == STAGE_CODE && cap != caps[0]) break;   // one CTA per SM, persistent
             HopTable t;
-            cudaError_t e = build_table(tmpl, nrb, nrb == STAGE_CODE ? sms : cap, t, dev, st, host, sta,
+            cudaError_t e = build_table(ctx, tmpl, nrb, nrb == STAGE_CODE ? sms : cap, t, dev, st, sta,
                                         band_order(prec));
             if (e == cudaSuccess) e = cudaStreamSynchronize(st);
             if (e != cudaSuccess) return e;
@@ -437,7 +435,7 @@ cudaError_t tune_hop_table(tm_ctx *ctx, int prec, int recon, const std::vector<B
     if (cache)
         tune_cache_store(ctx->tune_cache, ckey, "code" + std::to_string(best_nrb) + "-cap" + std::to_string(best_cap),
                          best);
-    cudaError_t e = build_table(tmpl, best_nrb, best_cap, out, dev, st, host, sta, band_order(prec));
+    cudaError_t e = build_table(ctx, tmpl, best_nrb, best_cap, out, dev, st, sta, band_order(prec));
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     return e;
 }
@@ -445,6 +443,30 @@ cudaError_t tune_hop_table(tm_ctx *ctx, int prec, int recon, const std::vector<B
 }  // namespace twm
 
 using namespace twm;
+
+cudaError_t HostTables::upload(void *dev, const void *src, size_t n, cudaStream_t s)
+{
+    constexpr size_t least = size_t(1) << 18;   // some tens of tables of 64 systems between waits
+    cudaError_t e = done_ ? cudaSuccess : cudaEventCreateWithFlags(&done_, cudaEventDisableTiming);
+    if (e == cudaSuccess && used_ + n > size_) {
+        e = cudaEventSynchronize(done_);
+        used_ = 0;
+        if (e == cudaSuccess && n > size_) {
+            if (host_) e = cudaFreeHost(host_);
+            host_ = nullptr;
+            size_ = 0;
+            if (e == cudaSuccess) e = cudaMallocHost(reinterpret_cast<void **>(&host_), std::max(n, least));
+            if (e == cudaSuccess) size_ = std::max(n, least);
+        }
+    }
+    if (e != cudaSuccess) return e;
+    memcpy(host_ + used_, src, n);
+    e = cudaMemcpyAsync(dev, host_ + used_, n, cudaMemcpyHostToDevice, s);
+    used_ += align256(n);
+    // the mark that the memory is waited for with, also where only some of several copies went out
+    const cudaError_t r = cudaEventRecord(done_, s);
+    return e == cudaSuccess ? r : e;
+}
 
 namespace {
 
@@ -526,7 +548,19 @@ extern "C" tm_status tm_Qtm_batch(tm_ctx *ctx, int nsys, const tm_gauge *const *
     }
     staged = staged && nrhs_max >= 2;
     cudaError_t e = cudaSuccess;
+    // Preparing a batch (link copies, tables, tuning) is not work that a graph
+    // may hold: a capturing stream takes only a batch that is in place.
+    auto refuse_capture = [&]() {
+        cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+        cudaError_t q = cudaStreamIsCapturing(s, &status);
+        if (q != cudaSuccess) (void)cudaGetLastError();
+        else if (status != cudaStreamCaptureStatusNone) q = cudaErrorStreamCaptureUnsupported;
+        return q;
+    };
     if (staged) {
+        for (auto *h : handles)
+            if (!h->links8 && e == cudaSuccess) e = refuse_capture();
+        if (e != cudaSuccess) return bcuda(ctx, e, "tm_Qtm_batch: a batch that is new to the context");
         // the staged hop is an optional candidate: without memory for its link
         // copies the batch runs with the gather hops alone
         for (auto *h : handles)
@@ -573,6 +607,8 @@ extern "C" tm_status tm_Qtm_batch(tm_ctx *ctx, int nsys, const tm_gauge *const *
         t.sa.roles = t.sa.smaps ? (1u << R_IN) | (1u << R_T) : 0u;
         dsys = static_cast<BSys *>(ctx->bq_tab.dsys);
     } else {
+        e = refuse_capture();
+        if (e != cudaSuccess) return bcuda(ctx, e, "tm_Qtm_batch: a batch that is new to the context");
         // the previous batch's launches may still read the buffer on another stream
         if (ctx->bq && ctx->bq_stream != s) {
             e = cudaStreamSynchronize(ctx->bq_stream);
@@ -621,8 +657,7 @@ extern "C" tm_status tm_Qtm_batch(tm_ctx *ctx, int nsys, const tm_gauge *const *
         c += align256(sizeof(BSys) * nsys);
         BGroup *dgrp = reinterpret_cast<BGroup *>(c);
         c += align256(sizeof(BGroup) * handles.size());
-        // pageable source: the copy has taken the data when the call returns
-        e = cudaMemcpyAsync(dsys, hs.data(), sizeof(BSys) * nsys, cudaMemcpyHostToDevice, s);
+        e = ctx->tables.upload(dsys, hs.data(), sizeof(BSys) * nsys, s);
         StageArgs sa{};
         if (staged && e == cudaSuccess) {
             // tensor maps of the two hop inputs of every system and of every group's links
@@ -641,9 +676,8 @@ extern "C" tm_status tm_Qtm_batch(tm_ctx *ctx, int nsys, const tm_gauge *const *
                 CUtensorMap *dsm = reinterpret_cast<CUtensorMap *>(c);
                 c += align256(sizeof(CUtensorMap) * nsmap);
                 CUtensorMap *dlm = reinterpret_cast<CUtensorMap *>(c);
-                e = cudaMemcpyAsync(dsm, hm.data(), sizeof(CUtensorMap) * nsmap, cudaMemcpyHostToDevice, s);
-                if (e == cudaSuccess)
-                    e = cudaMemcpyAsync(dlm, hl.data(), sizeof(CUtensorMap) * hl.size(), cudaMemcpyHostToDevice, s);
+                e = ctx->tables.upload(dsm, hm.data(), sizeof(CUtensorMap) * nsmap, s);
+                if (e == cudaSuccess) e = ctx->tables.upload(dlm, hl.data(), sizeof(CUtensorMap) * hl.size(), s);
                 sa.smaps = dsm;
                 sa.lmaps = dlm;
                 sa.status = ctx->dev_status;

@@ -35,6 +35,26 @@ class LinkPool {
     std::vector<std::pair<void *, size_t>> spare_;
 };
 
+// Small host tables on their way to the device: copied into pinned memory of
+// the context's own, so that the caller's copy may go away at once whether or
+// not the transfer has begun.  (A copy from pageable memory may be read later
+// where the GPU reads the host's pages itself.)  The pinned memory is reused
+// when the last transfer from it is done.
+class HostTables {
+  public:
+    ~HostTables()
+    {
+        if (done_) cudaEventSynchronize(done_), cudaEventDestroy(done_);
+        if (host_) cudaFreeHost(host_);
+    }
+    cudaError_t upload(void *dev, const void *src, size_t n, cudaStream_t s);
+
+  private:
+    char *host_ = nullptr;
+    size_t size_ = 0, used_ = 0;
+    cudaEvent_t done_ = nullptr;
+};
+
 struct tm_ctx {
     int device = 0;
     std::shared_ptr<LinkPool> pool = std::make_shared<LinkPool>();
@@ -66,6 +86,7 @@ struct tm_ctx {
     void *bq = nullptr;
     size_t bq_bytes = 0;
     std::vector<uintptr_t> bq_sig;
+    HostTables tables;
     cudaStream_t bq_stream = nullptr;
     struct {
         int nrb = 1, ngroups = 0;

@@ -43,3 +43,53 @@ def test_capture_before_the_first_qtm(dims):
     assert all(np.array_equal(c.unpack(o, vh, "f64").cpu().numpy(), w) for o, w in zip(outs, want))
     g.close()
     c.close()
+
+
+@pytest.mark.parametrize("prec,tol", [("f32", 1e-6), ("f64", 1e-13)])   # FP32 with the staged hop's tables, FP64 without
+def test_batch_in_a_capture(prec, tol):
+    """A batch that is new to the context (here: of a known shape, on other buffers) is refused by a capturing
+    stream and leaves the batch before it in place; one that is in place is captured and replays."""
+    from paper_1311_4521_gb300 import tmhop
+    dims, n = (8, 8, 8, 8), 3
+    vh = int(np.prod(dims)) // 2
+    U = F.gauge_field(dims, 951, "random")
+    psi = [F.gaussian_spinor(vh, 951, k) for k in range(2 * n)]
+    c = tmhop.Context(0)
+    g = c.gauge(dims, U, prec, 12 if prec == "f32" else 18)
+    ins = [c.pack(p, prec) for p in psi]
+    outs = [c.empty(vh, prec).zero_() for _ in psi]
+    want = [O.Qtm(dims, U, p, 0.16, 0.01) for p in psi]
+
+    def ok(ks):
+        return all(rel(c.unpack(outs[k], vh, prec).cpu().numpy(), want[k]) < tol for k in ks)
+
+    side = torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(side):
+        c.Qtm_batch([g] * n, outs[:n], ins[:n], 0.16, 0.01)
+        torch.cuda.synchronize()
+        assert ok(range(n))
+    refused, taken = torch.cuda.CUDAGraph(), torch.cuda.CUDAGraph()
+    with torch.cuda.graph(refused, stream=side):
+        with pytest.raises(tmhop.TmError):
+            c.Qtm_batch([g] * n, outs[n:], ins[n:], 0.16, 0.01)
+    with torch.cuda.graph(taken, stream=side):
+        c.Qtm_batch([g] * n, outs[:n], ins[:n], 0.16, 0.01)
+    for o in outs:
+        o.zero_()
+    torch.cuda.synchronize()
+    taken.replay()
+    torch.cuda.synchronize()
+    assert ok(range(n)) and not any(bool(o.any()) for o in outs[n:])
+    with torch.cuda.stream(side):
+        c.Qtm_batch([g] * n, outs[n:], ins[n:], 0.16, 0.01)
+        torch.cuda.synchronize()
+        assert ok(range(n, 2 * n))
+        for k in range(40):   # more tables than the pinned memory holds, buffers changing from call to call
+            o = outs[k % 2:] + outs[:k % 2]
+            c.Qtm_batch([g] * n, o[:n], ins[:n], 0.16, 0.01 + k)
+        c.Qtm_batch([g] * n, outs[:n], ins[:n], 0.16, 0.01)
+        torch.cuda.synchronize()
+        assert ok(range(n))
+    g.close()
+    c.close()
