@@ -183,9 +183,17 @@ tm_status tm_spinor_unpack(tm_ctx *ctx, long vh, const void *in_dev, double *out
  * and keeps no reference to U_dev.  Synchronous with respect to stream. */
 tm_status tm_gauge_create(tm_ctx *ctx, const int dims[4], const double *U_dev, int prec, int reconstruct,
                           const int bc[4], void *stream, tm_gauge **out);
-/* The context keeps the link buffers of the last destroyed handles (at most
- * two, together at most 1 GiB) for the next handles that fit, until it and
- * its last handle are destroyed.  A handle may outlive its context. */
+/* The same with the links in the caller's device memory mem_dev (16-byte
+ * aligned), of `bytes` bytes: at least the links, and for TM_F64 with all of
+ * tm_gauge_storage_bytes also their fixed-point copy.  The memory must stay
+ * until the handle is destroyed and every launch that uses it is done; a
+ * program that makes a handle per call spares itself the allocation, and the
+ * wait for the device that freeing one means. */
+tm_status tm_gauge_create_in(tm_ctx *ctx, const int dims[4], const double *U_dev, int prec, int reconstruct,
+                             const int bc[4], void *mem_dev, size_t bytes, void *stream, tm_gauge **out);
+/* Bytes that tm_gauge_create_in takes for such a handle; 0 if there is none. */
+size_t tm_gauge_storage_bytes(const int dims[4], int prec, int reconstruct);
+/* A handle may outlive its context. */
 void tm_gauge_destroy(tm_gauge *g);
 /* Bytes of device memory held by the handle's link storage.  A TM_F64 handle
  * also holds, memory permitting, a fixed-point copy of its links of the same

@@ -54,7 +54,9 @@ class _Packed:
 
 
 def _gauge(ctx, dims, U, prec, bc):
-    return ctx.gauge(dims, U.detach(), prec, RECON[prec], bc)
+    # a handle per call, used on the current stream only.  Forward and backward through Q_tm at 24^3x32 in FP32:
+    # 1.54 ms with an allocation and a free per handle
+    return tmhop.Gauge(ctx, dims, U.detach(), prec, RECON[prec], bc, torch_memory=True)
 
 
 class HoppingEO(torch.autograd.Function):

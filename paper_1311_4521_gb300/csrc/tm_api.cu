@@ -33,7 +33,7 @@ tm_status cuda_fail(tm_ctx *ctx, cudaError_t e, const char *where)
     } while (0)
 
 // Makes the fixed-point copy of an FP64 handle's links (tm_fix.cuh) in the
-// fx_copy_bytes + sizeof(int) bytes at fx; the handle keeps it unless some
+// fx_room bytes at fx; the handle keeps it unless some
 // link does not fit (the hops then use FP64 products).  Synchronises s.
 cudaError_t make_fx_links(tm_gauge *h, void *fx, cudaStream_t s)
 {
@@ -106,62 +106,6 @@ tm_status tm_ctx_reduce_buffer(tm_ctx *ctx, size_t bytes, void **ptr)
     }
     *ptr = ctx->red;
     return TM_OK;
-}
-
-cudaError_t LinkPool::take(size_t bytes, void **p, size_t *size)
-{
-    {
-        std::lock_guard<std::mutex> guard(lock_);
-        for (size_t k = 0; k < spare_.size(); ++k) {
-            if (spare_[k].second < bytes || spare_[k].second > 2 * bytes) continue;
-            *p = spare_[k].first;
-            *size = spare_[k].second;
-            spare_.erase(spare_.begin() + long(k));
-            const cudaError_t e = cudaDeviceSynchronize();
-            if (e != cudaSuccess) {
-                cudaFree(*p);
-                *p = nullptr;
-            }
-            return e;
-        }
-    }
-    cudaError_t e = cudaMalloc(p, bytes);
-    if (e == cudaErrorMemoryAllocation) {
-        (void)cudaGetLastError();   // not sticky
-        trim();
-        e = cudaMalloc(p, bytes);
-        if (e == cudaErrorMemoryAllocation) (void)cudaGetLastError();
-    }
-    *size = e == cudaSuccess ? bytes : 0;
-    return e;
-}
-
-void LinkPool::give(void *p, size_t size)
-{
-    std::vector<void *> drop;
-    {
-        std::lock_guard<std::mutex> guard(lock_);
-        if (size > kMost) {
-            drop.push_back(p);
-        } else {
-            size_t total = size;
-            for (auto &b : spare_) total += b.second;
-            while (!spare_.empty() && (spare_.size() >= 2 || total > kMost)) {   // the oldest go first
-                total -= spare_.front().second;
-                drop.push_back(spare_.front().first);
-                spare_.erase(spare_.begin());
-            }
-            spare_.push_back({p, size});
-        }
-    }
-    for (void *q : drop) cudaFree(q);
-}
-
-void LinkPool::trim()
-{
-    std::lock_guard<std::mutex> guard(lock_);
-    for (auto &b : spare_) cudaFree(b.first);
-    spare_.clear();
 }
 
 extern "C" {
@@ -296,19 +240,39 @@ tm_status tm_spinor_unpack(tm_ctx *ctx, long vh, const void *in_dev, double *out
     return TM_OK;
 }
 
-tm_status tm_gauge_create(tm_ctx *ctx, const int dims[4], const double *U_dev, int prec, int reconstruct,
-                          const int bc[4], void *stream, tm_gauge **out)
+}  // extern "C"
+
+static size_t link_bytes(const Geom &g, int prec, int reconstruct)
+{
+    return size_t(8) * link_nchunk(prec, reconstruct) * link_chunk_bytes(prec, reconstruct) * g.vh;
+}
+
+// Bytes for the fixed-point copy of an FP64 handle's links and its flag (make_fx_links).
+static size_t fx_room(const tm_gauge *h) { return align256(fx_copy_bytes(h) + sizeof(int)); }
+
+static tm_status bad_format(int prec, int reconstruct)
+{
+    if (!valid_prec(prec) || (reconstruct != 12 && reconstruct != 18)) return TM_ERR_ARG;
+    return prec == TM_F16 && reconstruct != 12 ? TM_ERR_UNSUPPORTED : TM_OK;
+}
+
+// A handle whose links live in memory of its own, or in the caller's (mem).
+static tm_status create_gauge(tm_ctx *ctx, const char *name, const int dims[4], const double *U_dev, int prec,
+                              int reconstruct, const int bc[4], void *mem, size_t mem_bytes, void *stream, tm_gauge **out)
 {
     if (!ctx) return TM_ERR_ARG;
-    if (!out || !dims || bad_ptr(U_dev) || !bc) return fail(ctx, TM_ERR_ARG, "tm_gauge_create: null or misaligned pointer");
+    auto refuse = [&](tm_status st, const char *why) { return tm_fail(ctx, st, std::string(name) + why); };
+    if (!out || !dims || bad_ptr(U_dev) || !bc) return refuse(TM_ERR_ARG, ": null or misaligned pointer");
     *out = nullptr;
-    if (!valid_prec(prec)) return fail(ctx, TM_ERR_ARG, "tm_gauge_create: bad precision");
-    if (reconstruct != 12 && reconstruct != 18) return fail(ctx, TM_ERR_ARG, "tm_gauge_create: reconstruct must be 12 or 18");
-    if (prec == TM_F16 && reconstruct != 12) return fail(ctx, TM_ERR_UNSUPPORTED, "tm_gauge_create: TM_F16 links need reconstruct 12");
+    if (const tm_status st = bad_format(prec, reconstruct))
+        return refuse(st, st == TM_ERR_UNSUPPORTED ? ": TM_F16 links need reconstruct 12"
+                          : valid_prec(prec)       ? ": reconstruct must be 12 or 18"
+                                                   : ": bad precision");
     for (int m = 0; m < 4; ++m)
-        if (bc[m] != 1 && bc[m] != -1) return fail(ctx, TM_ERR_ARG, "tm_gauge_create: bc entries must be +1 or -1");
+        if (bc[m] != 1 && bc[m] != -1) return refuse(TM_ERR_ARG, ": bc entries must be +1 or -1");
     Geom g;
-    if (!make_geom(dims, bc, g)) return fail(ctx, TM_ERR_ARG, "tm_gauge_create: extents must be even, >= 2, volume < 2^31");
+    if (!make_geom(dims, bc, g)) return refuse(TM_ERR_ARG, ": extents must be even, >= 2, volume < 2^31");
+    if (mem && mem_bytes < link_bytes(g, prec, reconstruct)) return refuse(TM_ERR_ARG, ": too little memory for the links");
     tm_gauge *h = new tm_gauge;
     h->ctx = ctx;
     memcpy(h->dims, dims, sizeof h->dims);
@@ -316,34 +280,71 @@ tm_status tm_gauge_create(tm_ctx *ctx, const int dims[4], const double *U_dev, i
     h->prec = prec;
     h->recon = reconstruct;
     h->geom = g;
-    h->bytes = size_t(8) * link_nchunk(prec, reconstruct) * link_chunk_bytes(prec, reconstruct) * g.vh;
-    h->pool = ctx->pool;
-    // the links, and for FP64 handles room for their fixed-point copy where there is memory
-    const size_t own = align256(h->bytes), copy = prec == TM_F64 ? fx_copy_bytes(h) + sizeof(int) : 0;
-    cudaError_t e = h->pool->take(own + copy, &h->links, &h->links_size);
-    const bool room = e == cudaSuccess;
-    if (e == cudaErrorMemoryAllocation && copy) e = h->pool->take(own, &h->links, &h->links_size);
-    if (e != cudaSuccess) {
-        delete h;
-        return cuda_fail(ctx, e, "cudaMalloc(links)");
+    h->bytes = link_bytes(g, prec, reconstruct);
+    // the links, and for FP64 handles their fixed-point copy where there is memory
+    const size_t copy = prec == TM_F64 ? fx_room(h) : 0;
+    void *fx = nullptr;
+    cudaError_t e = cudaSuccess;
+    if (mem) {
+        h->owns = false;
+        h->links = mem;
+        if (copy && mem_bytes >= align256(h->bytes) + copy) fx = static_cast<char *>(mem) + align256(h->bytes);
+    } else {
+        e = cudaMalloc(&h->links, h->bytes);
+        if (e == cudaSuccess && copy) {
+            e = cudaMalloc(&fx, copy);
+            if (e != cudaSuccess) fx = nullptr;
+            if (e == cudaErrorMemoryAllocation) {
+                (void)cudaGetLastError();   // not sticky
+                e = cudaSuccess;
+            }
+        }
     }
     cudaStream_t s = (cudaStream_t)stream;
-    e = launch_pack_gauge(g, prec, reconstruct, U_dev, h->links, s);
-    if (e == cudaSuccess && copy && room) e = make_fx_links(h, static_cast<char *>(h->links) + own, s);
+    if (e == cudaSuccess) e = launch_pack_gauge(g, prec, reconstruct, U_dev, h->links, s);
+    if (e == cudaSuccess && fx) e = make_fx_links(h, fx, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (h->owns && fx && !h->fx) cudaFree(fx);   // some link does not fit
     if (e != cudaSuccess) {
+        if (e == cudaErrorMemoryAllocation) (void)cudaGetLastError();   // not sticky
         tm_gauge_destroy(h);
-        return cuda_fail(ctx, e, "tm_gauge_create: pack");
+        return cuda_fail(ctx, e, name);
     }
     tm_apply_cached_map(ctx, h);
     *out = h;
     return TM_OK;
 }
 
+extern "C" {
+
+tm_status tm_gauge_create(tm_ctx *ctx, const int dims[4], const double *U_dev, int prec, int reconstruct,
+                          const int bc[4], void *stream, tm_gauge **out)
+{
+    return create_gauge(ctx, "tm_gauge_create", dims, U_dev, prec, reconstruct, bc, nullptr, 0, stream, out);
+}
+
+tm_status tm_gauge_create_in(tm_ctx *ctx, const int dims[4], const double *U_dev, int prec, int reconstruct,
+                             const int bc[4], void *mem_dev, size_t bytes, void *stream, tm_gauge **out)
+{
+    if (!ctx) return TM_ERR_ARG;
+    if (bad_ptr(mem_dev)) return fail(ctx, TM_ERR_ARG, "tm_gauge_create_in: null or misaligned memory");
+    return create_gauge(ctx, "tm_gauge_create_in", dims, U_dev, prec, reconstruct, bc, mem_dev, bytes, stream, out);
+}
+
+size_t tm_gauge_storage_bytes(const int dims[4], int prec, int reconstruct)
+{
+    const int bc[4] = {1, 1, 1, 1};
+    tm_gauge h;
+    if (!dims || bad_format(prec, reconstruct) != TM_OK || !make_geom(dims, bc, h.geom)) return 0;
+    h.recon = reconstruct;
+    return align256(link_bytes(h.geom, prec, reconstruct)) + (prec == TM_F64 ? fx_room(&h) : 0);
+}
+
 void tm_gauge_destroy(tm_gauge *g)
 {
     if (!g) return;
-    if (g->links) g->pool->give(g->links, g->links_size);
+    if (g->owns && g->links) cudaFree(g->links);
+    if (g->owns && g->fx) cudaFree(g->fx);
     if (g->links8) cudaFree(g->links8);
     delete g;
 }

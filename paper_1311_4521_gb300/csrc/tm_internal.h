@@ -5,35 +5,12 @@
 #include <cuda_runtime.h>
 
 #include <map>
-#include <memory>
-#include <mutex>
 #include <string>
 #include <utility>
 #include <vector>
 
 #include "tm_device.cuh"
 #include "tmhop.h"
-
-// Device buffers of destroyed gauge handles, kept for the next handle that
-// fits: a program that makes a handle per call (the autograd layer) spent
-// more time in cudaMalloc and cudaFree than in kernels (forward and backward
-// through Q_tm at 24^3x32 in FP32: 1.54 ms, 0.86 with the pool).  At most two buffers
-// of together at most kMost bytes; freed with the context and its last
-// handle, or when an allocation of a handle fails.  take() waits for the
-// device before it hands out a used buffer, since launches on any stream may
-// still read it (as cudaFree waited before).
-class LinkPool {
-  public:
-    ~LinkPool() { trim(); }
-    cudaError_t take(size_t bytes, void **p, size_t *size);
-    void give(void *p, size_t size);
-    void trim();
-
-  private:
-    static constexpr size_t kMost = size_t(1) << 30;
-    std::mutex lock_;
-    std::vector<std::pair<void *, size_t>> spare_;
-};
 
 // Small host tables on their way to the device: copied into pinned memory of
 // the context's own, so that the caller's copy may go away at once whether or
@@ -57,7 +34,6 @@ class HostTables {
 
 struct tm_ctx {
     int device = 0;
-    std::shared_ptr<LinkPool> pool = std::make_shared<LinkPool>();
     std::string err;
     void *scratch = nullptr;       // odd-parity temporaries of Q_tm and friends
     size_t scratch_bytes = 0;
@@ -155,8 +131,7 @@ struct tm_gauge {
     twm::Geom geom{};
     void *links = nullptr;
     size_t bytes = 0;
-    std::shared_ptr<LinkPool> pool;   // where links came from and goes back to
-    size_t links_size = 0;            // the buffer's size: links, then fx
+    bool owns = true;     // links and fx are the handle's own allocations, not the caller's memory (tm_gauge_create_in)
     twm::SiteMap map{};   // site-to-thread map of this lattice's hop launches (tm_gauge_tune)
     std::string map_name = "linear128";
     void *fx = nullptr;   // FP64 handles whose links fit (tm_fix.cuh): their fixed-point copy

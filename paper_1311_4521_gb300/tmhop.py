@@ -69,6 +69,8 @@ def _load() -> ctypes.CDLL:
         "tm_spinor_pack": ([P, L, P, P, I, P], I),
         "tm_spinor_unpack": ([P, L, P, P, I, P], I),
         "tm_gauge_create": ([P, I4, P, I, I, I4, P, ctypes.POINTER(P)], I),
+        "tm_gauge_create_in": ([P, I4, P, I, I, I4, P, S, P, ctypes.POINTER(P)], I),
+        "tm_gauge_storage_bytes": ([I4, I, I], S),
         "tm_gauge_destroy": ([P], None),
         "tm_gauge_bytes": ([P], S),
         "tm_hopping_eo": ([P, P, P, P, I, I, P], I),
@@ -183,6 +185,17 @@ def tm_gauge_create(ctx, dims, U_dev, prec, reconstruct, bc, stream=None) -> cty
     _check(ctx, lib.tm_gauge_create(ctx, _i4(dims), _ptr(U_dev), int(prec), int(reconstruct), _i4(bc),
                                     _stream(stream), ctypes.byref(h)))
     return h
+
+
+def tm_gauge_create_in(ctx, dims, U_dev, prec, reconstruct, bc, mem_dev, nbytes, stream=None) -> ctypes.c_void_p:
+    h = ctypes.c_void_p()
+    _check(ctx, lib.tm_gauge_create_in(ctx, _i4(dims), _ptr(U_dev), int(prec), int(reconstruct), _i4(bc),
+                                       _ptr(mem_dev), int(nbytes), _stream(stream), ctypes.byref(h)))
+    return h
+
+
+def tm_gauge_storage_bytes(dims, prec, reconstruct) -> int:
+    return int(lib.tm_gauge_storage_bytes(_i4(dims), int(prec), int(reconstruct)))
 
 
 def tm_gauge_destroy(g) -> None:
@@ -398,9 +411,14 @@ def tm_ctx_device_bytes(ctx) -> int:
 
 # ---- convenience layer over torch tensors -----------------------------------------
 class Gauge:
-    """A gauge handle: the library's packed copy of U in one precision."""
+    """A gauge handle: the library's packed copy of U in one precision.
 
-    def __init__(self, ctx: "Context", dims, U: torch.Tensor, prec="f64", reconstruct=18, bc=(-1, 1, 1, 1)):
+    ``torch_memory`` keeps it in memory of PyTorch's allocator instead of the handle's own, for a handle that is
+    used on one stream only, the current one at its creation (PyTorch hands the memory on in that stream's order,
+    so that neither making nor closing the handle allocates or waits for the device)."""
+
+    def __init__(self, ctx: "Context", dims, U: torch.Tensor, prec="f64", reconstruct=18, bc=(-1, 1, 1, 1),
+                 torch_memory=False):
         self.ctx = ctx
         self.dims = tuple(int(d) for d in dims)
         self.prec = PREC[prec] if isinstance(prec, str) else int(prec)
@@ -408,7 +426,18 @@ class Gauge:
         self.bc = tuple(bc)
         self.vh = int(np.prod(self.dims)) // 2
         Ur = _as_real_dev(U, ctx.device)
-        self.handle = tm_gauge_create(ctx.handle, self.dims, Ur, self.prec, self.reconstruct, self.bc)
+        self.memory = None
+        if torch_memory:
+            n = tm_gauge_storage_bytes(self.dims, self.prec, self.reconstruct)
+            try:
+                self.memory = torch.empty(n, dtype=torch.uint8, device=ctx.device) if n else None
+            except torch.OutOfMemoryError:   # the library's own allocation, which does without the FP64 copy
+                pass
+        if self.memory is None:
+            self.handle = tm_gauge_create(ctx.handle, self.dims, Ur, self.prec, self.reconstruct, self.bc)
+        else:
+            self.handle = tm_gauge_create_in(ctx.handle, self.dims, Ur, self.prec, self.reconstruct, self.bc,
+                                             self.memory, n)
 
     @property
     def nbytes(self) -> int:
@@ -418,6 +447,7 @@ class Gauge:
         if self.handle:
             tm_gauge_destroy(self.handle)
             self.handle = None
+            self.memory = None
 
     def __del__(self):
         try:
