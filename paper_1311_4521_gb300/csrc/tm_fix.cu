@@ -27,11 +27,13 @@ __global__ void __launch_bounds__(128) k_fx_links(unsigned vh, const double2 *__
     if (i >= vh) return;
     FxEntry u[9];
     bool ok = true;
+    unsigned bits = 0;   // of all entries, signs aside
 #pragma unroll
     for (int k = 0; k < NC; ++k) {
         const double2 v = ld_stream(links + (size_t(blk) * NC + k) * vh + i);
         // below 1 + 2^-20 and so finite
         ok = ok && (__double2hiint(v.x) & 0x7fffffff) < 0x3ff00001 && (__double2hiint(v.y) & 0x7fffffff) < 0x3ff00001;
+        bits |= unsigned((__double2hiint(v.x) | __double2hiint(v.y)) & 0x7fffffff) | unsigned(__double2loint(v.x) | __double2loint(v.y));
         fx_split(v.x, 1025u, 0u, u[k].x, u[k].y);
         fx_split(v.y, 1025u, 0u, u[k].z, u[k].w);
     }
@@ -40,7 +42,7 @@ __global__ void __launch_bounds__(128) k_fx_links(unsigned vh, const double2 *__
         u[7] = fx_minor(u[2], u[3], u[0], u[5]);
         u[8] = fx_minor(u[0], u[4], u[1], u[3]);
     }
-    if (!ok || !fx_link_ok(u)) {
+    if (!ok || !fx_link_ok(u, bits == 0)) {
         *unfit = 1;
         return;
     }

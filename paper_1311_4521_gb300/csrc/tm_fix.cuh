@@ -253,13 +253,14 @@ __device__ __forceinline__ FxEntry fx_minor(const FxEntry &a, const FxEntry &d, 
 
 // Whether a link (as limbs, each component below 1 + 2^-20) can be used: every
 // row's and column's sum of |re| + |im| at most 2.5 (sqrt(6) bounds it for a
-// unitary matrix), which bounds the sum of the 8 hops by 8 * 2.5 * 2^59 <
-// 2^63, and its largest component at least 1/16 (or all of them zero).
-__device__ __forceinline__ bool fx_link_ok(const FxEntry (&u)[9])
+// unitary matrix), which bounds a hop's product with a half-spinor below 2^58
+// by 2.5 * 2^58 and the sum of the 8 by 1.25 * 2^62 < 2^63, and its largest
+// component at least 1/16, or all of them zero (`zero`, by the bits of the
+// entries: limbs are zero below 2^-58 too).
+__device__ __forceinline__ bool fx_link_ok(const FxEntry (&u)[9], bool zero)
 {
     constexpr int most = int(2.5 * (1 << FX_LIMB));   // limbs are below 2^30, so three entries sum below 2^32.6
     bool ok = true;
-    unsigned bits = 0;
     int big = 0;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
@@ -270,11 +271,10 @@ __device__ __forceinline__ bool fx_link_ok(const FxEntry (&u)[9])
             row += unsigned(abs(r.x) + abs(r.z)) >> 1;
             col += unsigned(abs(c.x) + abs(c.z)) >> 1;
             big = max(big, max(abs(r.x), abs(r.z)));
-            bits |= unsigned(r.x | r.y | r.z | r.w);
         }
         ok = ok && row <= unsigned(most) / 2 && col <= unsigned(most) / 2;
     }
-    return ok && (big >= 1 << (FX_LIMB - 4) || bits == 0);
+    return ok && (big >= 1 << (FX_LIMB - 4) || zero);
 }
 
 // Staging of a hop's data: every thread copies its own neighbour site (12

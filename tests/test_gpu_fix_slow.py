@@ -72,3 +72,32 @@ def test_solve_with_a_source_of_wide_range(ctx, dims, bc, recon, inner):
     g.close()
     if lo:
         lo.close()
+
+
+@pytest.mark.parametrize("recon", [18, 12])
+@pytest.mark.parametrize("which", ["one", "all"])
+@pytest.mark.parametrize("scale", [1.3 * 2.0 ** -59, 1e-20, 1e-120, 0.0])
+def test_tiny_links_are_not_taken_for_zero(ctx, recon, which, scale):
+    """Links below the fixed-point unit act with what they are; links of exact zeros do nothing."""
+    dims = (4, 4, 4, 4)
+    V = 4 ** 4
+    U, psi = F.gauge_field(dims, 963, "random"), F.gaussian_spinor(V // 2, 963, 1)
+    rows = (slice(None), 7) if which == "one" else (slice(None), slice(None))
+    U[rows] = 0.0 if scale == 0.0 else U[rows] * scale
+    if recon == 12:
+        U[..., 2, :] = np.cross(U[..., 0, :], U[..., 1, :]).conj()
+    g, src = ctx.gauge(dims, U, "f64", recon), ctx.pack(psi, "f64")
+    for to in (0, 1):
+        got = ctx.unpack(ctx.hopping_eo(g, ctx.empty(V // 2, "f64"), src, to), V // 2, "f64").cpu().numpy()
+        want = O.hopping(dims, U, psi, to)
+        assert np.abs(got - want).max() <= 64 * EPS * np.abs(want).max()
+        for mu in range(4) if which == "one" else ():   # what enters through the changed links alone
+            only = np.zeros_like(U)
+            only[mu, 7] = U[mu, 7]
+            h = ctx.gauge(dims, only, "f64", recon)
+            got = ctx.unpack(ctx.hopping_eo(h, ctx.empty(V // 2, "f64"), src, to), V // 2, "f64").cpu().numpy()
+            want = O.hopping(dims, only, psi, to)
+            assert np.abs(got - want).max() <= 64 * EPS * np.abs(want).max()
+            assert bool(want.any()) == (scale != 0.0)
+            h.close()
+    g.close()
