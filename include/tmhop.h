@@ -556,9 +556,9 @@ tm_status tm_spinor_dot(tm_ctx *ctx, long vh, const void *a_dev, const void *b_d
  * alpha = 1 when alpha_dev is NULL.  Asynchronous on `stream`. */
 tm_status tm_scale_complex(tm_ctx *ctx, size_t n, double *z_dev, const double *alpha_dev, double c, void *stream);
 
-/* Bytes of device memory the context holds at this moment (its scratch,
- * solver workspace, staging slots, batch tables and reduction buffer; gauge
- * handles are counted by tm_gauge_bytes).  0 for a context that has not yet
+/* Bytes of device memory the context holds at this moment (its scratch, the
+ * fixed-point scratch of FP64 Q_tm, solver workspace, staging slots, batch
+ * tables and reduction buffer; gauge handles are counted by tm_gauge_bytes).  0 for a context that has not yet
  * allocated anything. */
 size_t tm_ctx_device_bytes(const tm_ctx *ctx);
 

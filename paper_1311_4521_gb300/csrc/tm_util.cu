@@ -207,7 +207,7 @@ tm_status tm_scale_complex(tm_ctx *ctx, size_t n, double *z_dev, const double *a
 size_t tm_ctx_device_bytes(const tm_ctx *ctx)
 {
     if (!ctx) return 0;
-    return ctx->scratch_bytes + ctx->ws_bytes + ctx->stage_bytes + ctx->bq_bytes + ctx->red_bytes;
+    return ctx->scratch_bytes + ctx->fx_scratch_bytes + ctx->ws_bytes + ctx->stage_bytes + ctx->bq_bytes + ctx->red_bytes;
 }
 
 }  // extern "C"

@@ -144,3 +144,17 @@ def test_handles_in_torch_memory_on_two_streams():
     for r, os in zip(ref, outs):
         assert all(torch.equal(r, o) for o in os)
     c.close()
+
+
+@pytest.mark.parametrize("dims", [(8, 8, 8, 8), (16, 16, 16, 16)])
+def test_device_bytes_count_the_fixed_point_scratch(dims):
+    from paper_1311_4521_gb300 import tmhop
+    c, vh = tmhop.Context(0), int(np.prod(dims)) // 2
+    g = c.gauge(dims, F.gauge_field(dims, 975, "near", 0.3), "f64", 18)
+    a, out = c.pack(F.gaussian_spinor(vh, 975, 1), "f64"), c.empty(vh, "f64")
+    assert tmhop.tm_ctx_device_bytes(c.handle) == 0
+    c.Qtm(g, out, a, 0.16, 0.01)
+    # two fields of 12 components of 16 bytes and a word a site, by blocks of 32 sites, and nothing else
+    assert tmhop.tm_ctx_device_bytes(c.handle) == 2 * vh * (12 * 16 + 4)
+    g.close()
+    c.close()
