@@ -46,6 +46,14 @@ cudaError_t make_fx_links(tm_gauge *h, void *fx, cudaStream_t s)
     return e;
 }
 
+// While it lives, this thread may allocate although a stream captures in
+// global mode; such a call would otherwise fail and end that capture.
+struct AllowAllocation {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    AllowAllocation() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~AllowAllocation() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
 bool valid_prec(int p) { return p == TM_F64 || p == TM_F32 || p == TM_F16 || p == TM_F64X; }
 
 }  // namespace
@@ -74,6 +82,8 @@ tm_status tm_qtm_scratch(tm_ctx *ctx, const tm_gauge *U, cudaStream_t s, void **
         const cudaError_t q = cudaStreamIsCapturing(s, &capture);
         if (q != cudaSuccess) (void)cudaGetLastError();   // the default stream while another one captures
         if (q == cudaSuccess && capture == cudaStreamCaptureStatusNone) {
+            // not part of a capture that this or another thread makes on another stream
+            const AllowAllocation allow;
             if (ctx->fx_scratch) {
                 const cudaError_t e = cudaFree(ctx->fx_scratch);
                 ctx->fx_scratch = nullptr;

@@ -93,3 +93,31 @@ def test_batch_in_a_capture(prec, tol):
         assert ok(range(n))
     g.close()
     c.close()
+
+
+def test_first_qtm_while_another_stream_captures():
+    """With the scratch of the other operators in place, a first FP64 Q_tm on a stream of its own leaves the capture
+    of another operator on another stream alone."""
+    from paper_1311_4521_gb300 import tmhop
+    dims = (8, 8, 8, 8)
+    vh = int(np.prod(dims)) // 2
+    U, psi = F.gauge_field(dims, 952, "random"), F.gaussian_spinor(vh, 952, 1)
+    c = tmhop.Context(0)
+    g, lo = c.gauge(dims, U, "f64", 18), c.gauge(dims, U, "f32", 12)
+    a, a32, out, out32 = c.pack(psi, "f64"), c.pack(psi, "f32"), c.empty(vh, "f64"), c.empty(vh, "f32")
+    c.Qnd(g, [c.empty(vh, "f64"), c.empty(vh, "f64")], [a, a], 0.16, 0.01, 0.02)
+    torch.cuda.synchronize()
+    graph, own = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    with torch.cuda.graph(graph):   # global mode
+        c.Qtm(lo, out32, a32, 0.16, 0.01)
+        tmhop.tm_Qtm(c.handle, g.handle, out, a, 0.16, 0.01, 1, own)
+    torch.cuda.synchronize()
+    out32.zero_()
+    graph.replay()
+    torch.cuda.synchronize()
+    want = O.Qtm(dims, U, psi, 0.16, 0.01)
+    assert rel(c.unpack(out, vh, "f64").cpu().numpy(), want) < 1e-13
+    assert rel(c.unpack(out32, vh, "f32").cpu().numpy(), want) < 1e-6
+    for h in (g, lo):
+        h.close()
+    c.close()
