@@ -255,7 +255,7 @@ cudaError_t qdagq(const tm_gauge *U, double kappa, double mu, const void *in, vo
                   bool iterate, const Work &w, int gate, cudaStream_t st)
 {
     double mut = 2.0 * kappa * mu;
-    if (U->fx) {   // t and q in fixed point
+    if (U->fx) {   // t in fixed point
         const CgFxArgs c{static_cast<double *>(w.y), static_cast<double *>(w.r), w.p, w.partials, w.s, gate};
         cudaError_t e = cudaSuccess;
         for (int stage = 0; stage < 4 && e == cudaSuccess; ++stage) {
@@ -485,12 +485,12 @@ extern "C" tm_status tm_cg_QdagQ(tm_ctx *ctx, const tm_gauge *U_hi, const tm_gau
     if (!w.mixed) S.Ul = U_hi;
 
     // workspace: FP64 ax, t_hi, q_hi (+ r in plain mode), inner r, p, q, t, y, partials, scalars
-    // (the hop temporaries t, q in fixed point where the handle has fixed-point links)
+    // (the hop temporary t in fixed point where the handle has fixed-point links)
     const bool fx_lo = S.Ul->fx != nullptr;
     const size_t f64 = spinor_bytes(w.vh, w.PH), flo = spinor_bytes(w.vh, w.P), fy = spinor_bytes(w.vh, w.PY);
-    const size_t ffx = fx_field_bytes(w.vh), tq_hi = U_hi->fx ? ffx : f64, tq = fx_lo ? ffx : flo;
+    const size_t ffx = fx_field_bytes(w.vh), t_hi = U_hi->fx ? ffx : f64, t_lo = fx_lo ? ffx : flo;
     const size_t nblk = blocks(w.vh, FX_BLOCK) + 1;   // the smallest CTA of a reducing launch
-    size_t need = align256(f64) + 2 * align256(tq_hi) + 2 * align256(flo) + 2 * align256(tq) + (fx_lo ? align256(ffx) : 0) +
+    size_t need = 2 * align256(f64) + align256(t_hi) + 3 * align256(flo) + align256(t_lo) + (fx_lo ? align256(ffx) : 0) +
                   (w.mixed ? align256(fy) : 0) + align256(nblk * sizeof(double)) + align256(sizeof(CgScalars));
     void *base = nullptr;
     tm_status st = tm_ctx_workspace(ctx, need, &base);
@@ -500,12 +500,12 @@ extern "C" tm_status tm_cg_QdagQ(tm_ctx *ctx, const tm_gauge *U_hi, const tm_gau
     w.x = x_dev;
     w.b = const_cast<void *>(b_dev);
     w.ax = take(f64);
-    w.t_hi = take(tq_hi);
-    w.q_hi = take(tq_hi);
+    w.t_hi = take(t_hi);
+    w.q_hi = take(f64);
     w.r = take(flo);
     w.p = take(flo);
-    w.q = take(tq);
-    w.t = take(tq);
+    w.q = take(flo);
+    w.t = take(t_lo);
     w.p_fx = fx_lo ? take(ffx) : nullptr;
     w.y = w.mixed ? take(fy) : x_dev;   // plain FP64: the update adds straight into x
     w.r_hi = w.r;

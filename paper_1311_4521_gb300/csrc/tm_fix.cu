@@ -34,8 +34,8 @@ __global__ void __launch_bounds__(128) k_fx_links(unsigned vh, const double2 *__
         // below 1 + 2^-20 and so finite
         ok = ok && (__double2hiint(v.x) & 0x7fffffff) < 0x3ff00001 && (__double2hiint(v.y) & 0x7fffffff) < 0x3ff00001;
         bits |= unsigned((__double2hiint(v.x) | __double2hiint(v.y)) & 0x7fffffff) | unsigned(__double2loint(v.x) | __double2loint(v.y));
-        fx_split(v.x, 1025u, 0u, u[k].x, u[k].y);
-        fx_split(v.y, 1025u, 0u, u[k].z, u[k].w);
+        fx_split_near(v.x, 1025u, u[k].x, u[k].y);
+        fx_split_near(v.y, 1025u, u[k].z, u[k].w);
     }
     if (RECON == 12 && ok) {
         u[6] = fx_minor(u[1], u[5], u[2], u[4]);
@@ -74,12 +74,14 @@ template <int PI> __global__ void __launch_bounds__(128) k_fx_field(unsigned vh,
 
 // The hop of k_hop / k_hop_io with fixed-point link products: input, re-read
 // input and output each packed FP64, canonical FP64 or (input and output) a
-// fixed-point field.
-template <int PI, int PX, int PO, int RECON, bool DAG, bool HASX, bool SIGNS>
+// fixed-point field; PR is the format of the input that sites left to FP64
+// products read (A.exact).
+template <int PI, int PR, int PX, int PO, int RECON, bool DAG, bool HASX, bool SIGNS>
 __global__ void __launch_bounds__(FX_BLOCK, TM_FX_MINB)
     k_fx_hop(const __grid_constant__ FxArgs A)
 {
     __shared__ int4 slots[FxStage<RECON>::WORDS * FX_BLOCK];
+    __shared__ unsigned words[12 * FX_BLOCK];
     const Geom &g = A.g;
     const SiteMap &m = A.m;
     // the map's CTAs of m.block threads, laid end to end; threads past the end repeat the last site
@@ -89,22 +91,18 @@ __global__ void __launch_bounds__(FX_BLOCK, TM_FX_MINB)
     const FxStage<RECON> st{slots + threadIdx.x};
     const int4 *x0 = HASX ? static_cast<const int4 *>(A.x) + (PX == F64C ? size_t(i) * 12 : size_t(i)) : nullptr;
     Spinor<double> acc, xs, o;
-    const bool slow = fx_hop_site<PI, RECON, DAG, SIGNS>(A, i, st, x0, PX == F64C ? 1 : g.vh, acc);
+    const FxSizes<FX_BLOCK> sizes(words);
+    const FxVerdict verdict = fx_hop_site<PI, RECON, DAG, SIGNS>(A, i, st, sizes, x0, PX == F64C ? 1 : g.vh, acc);
     if (HASX) st.wait();   // on every path: no thread leaves with copies to its slots under way
-    if (site >= g.vh) return;
-    if (slow) {
-        fx_slow_site<PI, PX, PO, RECON, DAG, HASX>(A, i);
-        return;
-    }
     if (HASX) st.site(xs);
     epilogue(A.k, acc, HASX ? &xs : nullptr, o);
-    SpinorIO<PO>::store(A.out, g.vh, i, o);
+    fx_finish<PR, PX, PO, RECON, DAG, HASX>(A, i, site < g.vh, verdict, o);
 }
 
 // The same hop with the 8 hops of a site dealt out to four warps, one
 // direction each, for lattices whose sites do not fill the GPU: a CTA covers
-// 32 sites.  The warps' integer sums meet in shared memory, then warp w
-// finishes spin w.  The site map is not used (results do not depend on it).
+// 32 sites.  The warps' integer sums, and the sums of absolute values, meet in
+// shared memory, then warp w finishes spin w.  The site map is not used (results do not depend on it).
 constexpr int FX_SPLIT = 128;
 template <int RECON> constexpr size_t fx_split_bytes() { return sizeof(int4) * FxStage<RECON, FX_SPLIT>::WORDS * FX_SPLIT; }
 
@@ -113,6 +111,7 @@ __global__ void __launch_bounds__(FX_SPLIT, 3) k_fx_hop_split(const __grid_const
 {
     extern __shared__ int4 dyn[];
     __shared__ int4 info[FX_SPLIT];
+    __shared__ unsigned words[12 * FX_SPLIT];   // [12][4 directions][32]
     const Geom &g = A.g;
     const unsigned vh = g.vh, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const unsigned site = blockIdx.x * 32 + lane, i = min(site, vh - 1);
@@ -121,13 +120,9 @@ __global__ void __launch_bounds__(FX_SPLIT, 3) k_fx_hop_split(const __grid_const
     neighbours(g, A.p, i, n);
     const FxLinks<RECON> src{A.fx, vh, i, A.p};
     FxSum t;
-#pragma unroll
-    for (int s = 0; s < 4; ++s)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) t.re[s][c] = t.im[s][c] = 0;
-    FxRange r;
     unsigned long long d = 0;
-    t.e = -5000;
+    t.clear(FX_LOWEST_E);
+    const FxSizes<FX_SPLIT> sizes(words);
     switch (w) {
     case 0: fx_start<PI, 0>(g, n, src, A.in, st); break;
     case 1: fx_start<PI, 2>(g, n, src, A.in, st); break;
@@ -144,24 +139,21 @@ __global__ void __launch_bounds__(FX_SPLIT, 3) k_fx_hop_split(const __grid_const
     bool slow = false;
     if constexpr (PI == FXF) slow = fx_exponents(n, A.in, vh, t.e, d);
     switch (w) {
-    case 0: fx_hops<PI, DAG, 0, 1, SIGNS>(g, n, src, A.in, st, nullptr, 0, d, t, r); break;
-    case 1: fx_hops<PI, DAG, 2, 3, SIGNS>(g, n, src, A.in, st, nullptr, 0, d, t, r); break;
-    case 2: fx_hops<PI, DAG, 4, 5, SIGNS>(g, n, src, A.in, st, nullptr, 0, d, t, r); break;
-    default: fx_hops<PI, DAG, 6, 7, SIGNS>(g, n, src, A.in, st, nullptr, 0, d, t, r);
+    case 0: fx_hops<PI, DAG, 0, 1, SIGNS>(g, n, src, A.in, st, nullptr, 0, d, t, sizes, slow); break;
+    case 1: fx_hops<PI, DAG, 2, 3, SIGNS>(g, n, src, A.in, st, nullptr, 0, d, t, sizes, slow); break;
+    case 2: fx_hops<PI, DAG, 4, 5, SIGNS>(g, n, src, A.in, st, nullptr, 0, d, t, sizes, slow); break;
+    default: fx_hops<PI, DAG, 6, 7, SIGNS>(g, n, src, A.in, st, nullptr, 0, d, t, sizes, slow);
     }
     if constexpr (PI != FXF) {   // the directions' exponents and ranges meet first
-        info[threadIdx.x] = make_int4(t.e, int(r.fmax), int(r.fmin), r.bad);
+        info[threadIdx.x] = make_int4(t.e, slow, 0, 0);
         __syncthreads();
         const int own = t.e;
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
             const int4 q = info[32 * v + lane];
             t.e = max(t.e, q.x);
-            r.fmax = max(r.fmax, unsigned(q.y));
-            r.fmin = min(r.fmin, unsigned(q.z));
-            r.bad = r.bad || q.w;
+            slow = slow || q.y;
         }
-        slow = fx_range_slow(r);
 #pragma unroll
         for (int s = 0; s < 4; ++s)
 #pragma unroll
@@ -169,6 +161,7 @@ __global__ void __launch_bounds__(FX_SPLIT, 3) k_fx_hop_split(const __grid_const
                 t.re[s][c] = fx_sar(t.re[s][c], t.e - own);
                 t.im[s][c] = fx_sar(t.im[s][c], t.e - own);
             }
+        sizes.sar(t.e - own);
     } else {
         __syncthreads();   // every warp has read its staged words
     }
@@ -186,42 +179,55 @@ __global__ void __launch_bounds__(FX_SPLIT, 3) k_fx_hop_split(const __grid_const
     const cpx<double> a = up ? cpx<double>{A.k.d[0], A.k.d[1]} : cpx<double>{A.k.d[2], A.k.d[3]};
     const cpx<double> b = up ? cpx<double>{A.k.d[4], A.k.d[5]} : cpx<double>{A.k.d[6], A.k.d[7]};
     cpx<double> o[3];
+    unsigned least2 = 0xffffffffu;   // of this warp's spin, re and im
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
         const long long *q = part + (6 * w + 2 * c) * FX_SPLIT + lane;
         const long long re = q[0] + q[32] + q[64] + q[96];
         const long long im = q[FX_SPLIT] + q[FX_SPLIT + 32] + q[FX_SPLIT + 64] + q[FX_SPLIT + 96];
         const cpx<double> hop = {fx_to_double(re, t.e, bits), fx_to_double(im, t.e, bits)};
+        const volatile unsigned *z = words + (3 * w + c) * FX_SPLIT + lane;
+        least2 = __vminu2(least2, z[0] + z[32] + z[64] + z[96]);
         o[c] = A.k.unit ? (up ? hop : -hop) : a * hop;
         if (HASX) o[c] = cmadd(b, cpx<double>{x[c].x, x[c].y}, o[c]);
     }
+    // the spins' ranges and smallest sums meet; then all know what is to be done
+    int least = int(min(least2 & 0xffffu, least2 >> 16));
+    unsigned m = 0, any = 0;
+    if (PO == FXF)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) fx_range_of(o[c], m, any);
+    __syncthreads();
+    info[threadIdx.x] = make_int4(int(m), int(any), least, 0);
+    __syncthreads();
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+        const int4 q = info[32 * v + lane];
+        m = max(m, unsigned(q.x));
+        any |= unsigned(q.y);
+        least = min(least, q.z);
+    }
+    const FxVerdict verdict(slow, least, t.e, bits);
+    bool again = verdict.least < FX_LEAST;
     if constexpr (PO == FXF) {
-        unsigned m = 0, lowest = 0xffffffffu, any = 0;
-#pragma unroll
-        for (int c = 0; c < 3; ++c) fx_range_of(o[c], m, lowest, any);
-        __syncthreads();
-        info[threadIdx.x] = make_int4(int(m), int(lowest), int(any), 0);
-        __syncthreads();
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            const int4 q = info[32 * v + lane];
-            m = max(m, unsigned(q.x));
-            lowest = min(lowest, unsigned(q.y));
-            any |= unsigned(q.z);
-        }
+        const FxSite f(m, any);
         if (site < vh && !slow) {
-            const FxSite f(m, lowest, any);
 #pragma unroll
             for (int c = 0; c < 3; ++c) f.store(A.out, i, 3 * w + c, o[c]);
             if (w == 0) f.store_word(A.out, vh, i);
         }
+        again = again || !fx_stores(A, float(verdict.least), verdict.e, f);
     } else if (site < vh && !slow) {
         double2 *q = static_cast<double2 *>(A.out);
 #pragma unroll
         for (int c = 0; c < 3; ++c)
             st_stream(PO == F64C ? q + size_t(i) * 12 + 3 * w + c : q + size_t(3 * w + c) * vh + i, make_double2(o[c].re, o[c].im));
     }
-    if (slow && w == 0 && site < vh) fx_slow_site<PI, PX, PO, RECON, DAG, HASX>(A, i);
+    __syncthreads();   // the spins' stores come before what may replace them
+    if (w == 0) {
+        const int todo = site >= vh ? FX_DONE : slow ? FX_SLOW : again ? FX_CHECK : FX_DONE;
+        if (__any_sync(0xffffffffu, todo != FX_DONE)) fx_again<PI, PX, PO, RECON, DAG, HASX>(A, i, verdict.e, todo);
+    }
 }
 
 // Lattices up to this many sites per parity take the split hop: as many as
@@ -233,18 +239,19 @@ __global__ void __launch_bounds__(FX_SPLIT, 3) k_fx_hop_split(const __grid_const
 #define TM_FX_SPLIT_SITES 14592
 #endif
 
-template <int PI, int PX, int PO, int RECON, bool DAG, bool HASX>
+template <int PI, int PR, int PX, int PO, int RECON, bool DAG, bool HASX>
 static cudaError_t fx_launch(const FxArgs &A, cudaStream_t s)
 {
     const unsigned vh = A.g.vh;
     const bool signs = A.g.anti[1] || A.g.anti[2] || A.g.anti[3];
     if (vh <= TM_FX_SPLIT_SITES) {
+        static_assert(!(HASX && PO == FXF), "fx_stores takes the hop alone");
         auto kern = k_fx_hop_split<PI, PX, PO, RECON, DAG, HASX, true>;
         const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(fx_split_bytes<RECON>()));
         if (e != cudaSuccess) return e;
         kern<<<(vh + 31) / 32, FX_SPLIT, fx_split_bytes<RECON>(), s>>>(A);
     } else {
-        auto kern = signs ? k_fx_hop<PI, PX, PO, RECON, DAG, HASX, true> : k_fx_hop<PI, PX, PO, RECON, DAG, HASX, false>;
+        auto kern = signs ? k_fx_hop<PI, PR, PX, PO, RECON, DAG, HASX, true> : k_fx_hop<PI, PR, PX, PO, RECON, DAG, HASX, false>;
         kern<<<(vh + FX_BLOCK - 1) / FX_BLOCK, FX_BLOCK, 0, s>>>(A);
     }
     return cudaGetLastError();
@@ -254,9 +261,9 @@ template <int RECON>
 static cudaError_t launch_f64_fields(const tm_gauge *U, bool dag, int p, const void *in, void *out, const void *x, const Coef &k,
                           cudaStream_t s, const SiteMap &m)
 {
-    const FxArgs A{U->geom, m, k, p, static_cast<const FxEntry *>(U->fx), static_cast<const double2 *>(U->links), in, x, out};
-    if (dag) return x ? fx_launch<F64, F64, F64, RECON, true, true>(A, s) : fx_launch<F64, F64, F64, RECON, true, false>(A, s);
-    return x ? fx_launch<F64, F64, F64, RECON, false, true>(A, s) : fx_launch<F64, F64, F64, RECON, false, false>(A, s);
+    const FxArgs A(U->geom, m, k, p, U->fx, U->links, in, x, out, in);
+    if (dag) return x ? fx_launch<F64, F64, F64, F64, RECON, true, true>(A, s) : fx_launch<F64, F64, F64, F64, RECON, true, false>(A, s);
+    return x ? fx_launch<F64, F64, F64, F64, RECON, false, true>(A, s) : fx_launch<F64, F64, F64, F64, RECON, false, false>(A, s);
 }
 
 cudaError_t launch_fx_hop(const tm_gauge *U, bool dag, int out_parity, const void *in, void *out, const void *x,
@@ -274,18 +281,14 @@ template <int PI, int RECON>
 static cudaError_t fx_qtm(const tm_gauge *U, bool stage_b, const void *in, void *tmp, void *out, const Coef &k, cudaStream_t s)
 {
     const Geom &g = U->geom;
-    FxArgs A{g, U->map, k, stage_b ? 0 : 1, static_cast<const FxEntry *>(U->fx), static_cast<const double2 *>(U->links), in, nullptr, tmp};
-    if (stage_b) {
-        A.in = tmp;
-        A.x = in;
-        A.out = out;
-        return fx_launch<FXF, PI, PI, RECON, false, true>(A, s);
-    }
-    if (g.vh <= TM_FX_SPLIT_SITES) return fx_launch<PI, F64, FXF, RECON, false, false>(A, s);
+    auto args = [&](const void *input, const void *x, void *output, const void *exact) {
+        return FxArgs(g, U->map, k, stage_b ? 0 : 1, U->fx, U->links, input, x, output, exact);
+    };
+    if (stage_b) return fx_launch<FXF, FXF, PI, PI, RECON, false, true>(args(tmp, in, out, tmp), s);
+    if (g.vh <= TM_FX_SPLIT_SITES) return fx_launch<PI, PI, F64, FXF, RECON, false, false>(args(in, nullptr, tmp, in), s);
     void *even = static_cast<char *>(tmp) + align256(fx_field_bytes(g.vh));
     k_fx_field<PI><<<(g.vh + 127) / 128, 128, 0, s>>>(g.vh, in, even);
-    A.in = even;
-    return fx_launch<FXF, F64, FXF, RECON, false, false>(A, s);
+    return fx_launch<FXF, PI, F64, FXF, RECON, false, false>(args(even, nullptr, tmp, in), s);
 }
 
 cudaError_t launch_fx_qtm(const tm_gauge *U, bool canonical, bool stage_b, const void *in, void *tmp, void *out,
