@@ -198,10 +198,12 @@ void tm_gauge_destroy(tm_gauge *g);
 /* Bytes of device memory held by the handle's link storage.  A TM_F64 handle
  * also holds, memory permitting, a fixed-point copy of its links of the same
  * size, which its hop launches (tm_hopping_eo, tm_Qtm, tm_Qtm_host, tm_force,
- * tm_solve_eo) multiply with on the integer units, about four times as fast
- * as in FP64 and no less exact; a field with a link that is far from SU(3)
- * (|re|+|im| of a row or column above 2.5, an entry above 1, none above 1/16)
- * has none and uses FP64 products throughout. */
+ * tm_solve_eo, tm_cg_QdagQ) multiply with on the integer units, about four
+ * times as fast as in FP64 and no less exact: an output component whose error
+ * that way could exceed what FP64 products leave, relative to the absolute
+ * products that enter it, is computed with those.  A field with a link that
+ * is far from SU(3) (|re|+|im| of a row or column above 2.5, an entry above 1,
+ * none above 1/16) has no copy and uses FP64 products throughout. */
 size_t tm_gauge_bytes(const tm_gauge *g);
 
 /* Site-to-thread maps of the hop launches (tm_hopping_eo, tm_Qtm, tm_force,

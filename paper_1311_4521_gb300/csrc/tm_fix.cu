@@ -4,7 +4,7 @@
 #include "tm_internal.h"
 
 // Resident CTAs of 64 threads per SM the fixed-point hops are compiled for:
-// 6 (168 registers) measured fastest at 32^3x64: Q_tm 0.80 ms against 0.94
+// 6 (168 registers) measured fastest at 32^3x64: when chosen, Q_tm 0.80 ms against 0.94
 // (4) and 0.96 (7, whose 128 registers spill); the hop on FP64 fields 0.47
 // against 0.56 ms (4).
 #ifndef TM_FX_MINB
@@ -231,10 +231,12 @@ __global__ void __launch_bounds__(FX_SPLIT, 3) k_fx_hop_split(const __grid_const
 }
 
 // Lattices up to this many sites per parity take the split hop: as many as
-// three of its CTAs per SM hold at once (3 x 152 x 32).  Measured, Q_tm whole
-// / split in us: 8^4 31 / 18, 8^3x16 31 / 20, 10^3x20 33 / 27, 12^3x24 37 /
-// 43, 16^4 41 / 59 (more warps, but each repeats the neighbour arithmetic and
-// the sums cross shared memory).
+// three of its CTAs per SM hold at once (3 x 152 x 32).  Measured in a graph,
+// Q_tm whole / split in us: 8^4 27 / 16, 8^3x16 29 / 19, 10^3x20 32 / 26,
+// 12^3x16 (13,824 sites) 30 / 27, 14x14x10x16 (15,680) 29 / 37, 12^3x24 34 /
+// 40, 16^4 40 / 56 (more warps, but each repeats the neighbour arithmetic and
+// the sums cross shared memory); with 12-real links 43 / 35 and 40 / 49 on
+// either side of the line.
 #ifndef TM_FX_SPLIT_SITES
 #define TM_FX_SPLIT_SITES 14592
 #endif

@@ -25,13 +25,12 @@
 // against 64-bit and longer arithmetic, Q_tm is off by 1.2e-16 (1.3e-16 with
 // FP64 products).
 //
-// Measured (32^3x64, 18-real links): Q_tm 3.04 -> 0.77 ms, one hop 1.52 ->
-// 0.47 ms; 8^4, split over warps: Q_tm 65 -> 18 us.  Launch B moves 4.9 TB/s, 0.73 of the
-// measured copy bandwidth; its multiply-add pipe is busy 57 % of the time.
+// Measured (32^3x64, 18-real links, against FP64 products): Q_tm 3.04 -> 0.78
+// ms, one hop 1.52 -> 0.49 ms; 8^4, split over warps: Q_tm 65 -> 19 us.
 // What it took beyond the integers (Q_tm at 32^3x64): multiply-adds from
 // plain C, not inline PTX 1.36 -> 1.02 ms; neighbours and links staged by
 // cp.async one hop ahead, 12 warps per SM, 0.87; the fallback called with
-// two words instead of with the site's sum 0.80.
+// few words instead of with the site's sum 0.80.
 #pragma once
 
 #include <cmath>
@@ -821,9 +820,10 @@ enum { FX_DONE = 0, FX_CHECK = 1, FX_SLOW = 2 };
 // it to be stored so).  FX_SLOW and the others: computed with FP64 products,
 // from the input to the stored result.  A call whose arguments are few words:
 // passing the site's sum in and out cost 7 % of the kernel.  Up to 4 sites are
-// checked by the whole warp: alone, a lane's 8 hops are a chain of some 5 us,
-// 28 us of Q_tm on 16^4, where some warp always has such a site; more of them
-// (a field with components of exactly zero) by a lane each.
+// checked by the whole warp: alone, a lane's 8 hops are a chain of several us
+// that every launch had to wait for somewhere (Q_tm on 16^4 69 us, now 40; on
+// 8^4 45, now 16); more of them (a field with components of exactly zero) by
+// a lane each.
 template <int PR, int PX, int PO, int RECON, bool DAG, bool HASX>
 __device__ __noinline__ void fx_again(const FxArgs &A, unsigned i, int e, int todo)
 {

@@ -189,12 +189,15 @@ __global__ void __launch_bounds__(128, TM_HOP_MINB(F64X))
 
 // Lattices that take it: up to 16000 sites per parity, and for 18-real links
 // from the second wave of the whole hop (more than 2 x 152 CTAs of 128) to
-// 160000.  Measured, Q_tm and the result's unpacking, whole / split in us,
-// 18-real links: 8^4 61 / 33, 16^3x32 133 / 107, 20^3x40 252 / 241; 12-real,
-// whose warps each rebuild the rows they need: 10^3x20 75 / 46, 12^3x24 82 /
-// 82, 16^4 86 / 114.  Between the two ranges the whole hop is one wave of 23
-// to 25 us: a hop 14^3x28 25.0 / 26.1; 12^3x24 with unpacking, one call
-// after another, 36.9 on every run against 30, 37 and 41.
+// 160000.  In a graph, Q_tm whole / split in us, 18-real and 12-real links
+// (whose warps each rebuild the rows they need): 8^4 51 / 17 and 70 / 25;
+// 13,824 sites 50 / 21 and 65 / 33; 15,680 51 / 37 and 65 / 62; 17,280 52 / 38
+// and 66 / 65 with the hop at 29.4 / 31.4; 40,960 65 / 58 and 76 / 107;
+// 128,000 185 / 163; 160,000 210 / 204; 221,184 272 / 274.  Between the two
+// ranges the whole hop is one wave of 24 to 26 us, and the split one ahead of
+// it in a graph (20,736: 25 / 18) but not in turn with other launches:
+// 12^3x24 and the unpacking of its result, one call after another, 36.9 on
+// every run against 30, 37 and 41.
 inline bool f64x_split(int recon, unsigned vh)
 {
     return vh <= 16000 || (recon == 18 && vh > 2 * 152 * 128 && vh <= 160000);
