@@ -196,7 +196,8 @@ size_t tm_gauge_storage_bytes(const int dims[4], int prec, int reconstruct);
 /* A handle may outlive its context. */
 void tm_gauge_destroy(tm_gauge *g);
 /* Bytes of device memory held by the handle's link storage.  A TM_F64 handle
- * also holds, memory permitting, a fixed-point copy of its links of the same
+ * also holds, where half of the device's memory stays free beside it and
+ * tm_ctx_set_fixed_point has not said otherwise, a fixed-point copy of its links of the same
  * size, which its hop launches (tm_hopping_eo, tm_Qtm, tm_Qtm_host, tm_force,
  * tm_solve_eo, tm_cg_QdagQ) multiply with on the integer units, about four
  * times as fast as in FP64 and no less exact: an output component whose error
@@ -205,6 +206,9 @@ void tm_gauge_destroy(tm_gauge *g);
  * is far from SU(3) (|re|+|im| of a row or column above 2.5, an entry above 1,
  * none above 1/16) has no copy and uses FP64 products throughout. */
 size_t tm_gauge_bytes(const tm_gauge *g);
+/* Whether TM_F64 handles that ctx makes from now on get that copy (on = 1, the
+ * default) or use FP64 products throughout in half the memory (0). */
+tm_status tm_ctx_set_fixed_point(tm_ctx *ctx, int on);
 
 /* Site-to-thread maps of the hop launches (tm_hopping_eo, tm_Qtm, tm_force,
  * tm_solve_eo) on the handle's lattice.  "linear<B>" gives CTAs of B threads

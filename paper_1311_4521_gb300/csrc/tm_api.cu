@@ -1,5 +1,6 @@
 // tm_api.cu -- the C ABI of include/tmhop.h: contexts, gauge handles,
 // packed fields, the hopping matrix and Q_tm.
+#include <algorithm>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -179,6 +180,13 @@ tm_status tm_ctx_check(tm_ctx *ctx)
     return TM_OK;
 }
 
+tm_status tm_ctx_set_fixed_point(tm_ctx *ctx, int on)
+{
+    if (!ctx) return TM_ERR_ARG;
+    ctx->fixed_point = on ? 1 : 0;
+    return TM_OK;
+}
+
 tm_status tm_ctx_set_autotune(tm_ctx *ctx, int on)
 {
     if (!ctx) return TM_ERR_ARG;
@@ -260,6 +268,22 @@ static size_t link_bytes(const Geom &g, int prec, int reconstruct)
 // Bytes for the fixed-point copy of an FP64 handle's links and its flag (make_fx_links).
 static size_t fx_room(const tm_gauge *h) { return align256(fx_copy_bytes(h) + sizeof(int)); }
 
+// Whether there is memory for the fixed-point copy of h's links beside what a
+// program may still need: after it at least half of the device's memory is
+// free, and 3 KiB per site of one parity, more than a solve on the lattice
+// takes (workspace 1.6 KiB, of the full system another 1.3).  So the copies of
+// all handles together never take the second half, and a lattice whose solve
+// fits without a copy does not lose it to one.
+static bool fx_fits(const tm_gauge *h)
+{
+    size_t left = 0, total = 0;
+    if (cudaMemGetInfo(&left, &total) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    return left >= fx_room(h) + std::max(total / 2, size_t(3072) * h->geom.vh);
+}
+
 static tm_status bad_format(int prec, int reconstruct)
 {
     if (!valid_prec(prec) || (reconstruct != 12 && reconstruct != 18)) return TM_ERR_ARG;
@@ -292,7 +316,7 @@ static tm_status create_gauge(tm_ctx *ctx, const char *name, const int dims[4], 
     h->geom = g;
     h->bytes = link_bytes(g, prec, reconstruct);
     // the links, and for FP64 handles their fixed-point copy where there is memory
-    const size_t copy = prec == TM_F64 ? fx_room(h) : 0;
+    const size_t copy = prec == TM_F64 && ctx->fixed_point ? fx_room(h) : 0;
     void *fx = nullptr;
     cudaError_t e = cudaSuccess;
     if (mem) {
@@ -301,7 +325,7 @@ static tm_status create_gauge(tm_ctx *ctx, const char *name, const int dims[4], 
         if (copy && mem_bytes >= align256(h->bytes) + copy) fx = static_cast<char *>(mem) + align256(h->bytes);
     } else {
         e = cudaMalloc(&h->links, h->bytes);
-        if (e == cudaSuccess && copy) {
+        if (e == cudaSuccess && copy && fx_fits(h)) {
             e = cudaMalloc(&fx, copy);
             if (e != cudaSuccess) fx = nullptr;
             if (e == cudaErrorMemoryAllocation) {

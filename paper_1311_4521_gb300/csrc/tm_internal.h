@@ -45,6 +45,7 @@ struct tm_ctx {
     size_t ws_bytes = 0;
     void *red = nullptr;             // partial sums of tm_spinor_dot (grow-only)
     size_t red_bytes = 0;
+    int fixed_point = 1;             // FP64 handles get a fixed-point copy of their links (tm_ctx_set_fixed_point)
     int autotune = 1;                // time launch configurations on first use
     int batch_code = -1;             // forced batched-hop configuration (tm_ctx_set_batch_config), -1 = tuned
     unsigned batch_cap = 0;          // and its persistent CTA cap (0: one CTA per work item)

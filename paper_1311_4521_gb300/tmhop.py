@@ -78,6 +78,7 @@ def _load() -> ctypes.CDLL:
         "tm_Qtm_noalloc": ([P, P, P, P, D, D, I, P], I),
         "tm_cg_QdagQ": ([P, P, P, P, P, ctypes.POINTER(CgParams), ctypes.POINTER(CgInfo), P], I),
         "tm_ctx_set_autotune": ([P, I], I),
+        "tm_ctx_set_fixed_point": ([P, I], I),
         "tm_ctx_tune_report": ([P, ctypes.c_char_p, ctypes.c_size_t], ctypes.c_size_t),
         "tm_force": ([P, P, P, P, D, D, I, P], I),
         "tm_force_ex": ([P, P, P, P, D, D, I, I, P], I),
@@ -243,6 +244,11 @@ def tm_force(ctx, U, F_dev, X_e_dev, kappa, mu, mode=TM_FORCE_SU3, stream=None):
 def tm_force_ex(ctx, U, F_dev, X_e_dev, kappa, mu, mode=TM_FORCE_SU3, scheme=TM_FORCE_OWNER, stream=None):
     _check(ctx, lib.tm_force_ex(ctx, U, _ptr(F_dev), _ptr(X_e_dev), float(kappa), float(mu), int(mode), int(scheme),
                                 _stream(stream)))
+
+
+def tm_ctx_set_fixed_point(ctx, on: bool) -> None:
+    """Whether FP64 handles made from now on get a fixed-point copy of their links (the default) or do without."""
+    _check(ctx, lib.tm_ctx_set_fixed_point(ctx, int(bool(on))))
 
 
 def tm_ctx_set_autotune(ctx, on: bool) -> None:

@@ -158,3 +158,35 @@ def test_device_bytes_count_the_fixed_point_scratch(dims):
     assert tmhop.tm_ctx_device_bytes(c.handle) == 2 * vh * (12 * 16 + 4)
     g.close()
     c.close()
+
+
+def test_fixed_point_copies_can_be_refused_and_leave_room():
+    from paper_1311_4521_gb300 import tmhop
+    c = tmhop.Context(0)
+    U, psi = F.gauge_field(DIMS, 976, "random"), F.gaussian_spinor(VH, 976, 1)
+    a, want, links = c.pack(psi, "f64"), O.Qtm(DIMS, U, psi, 0.16, 0.01), 8 * VH * 144
+
+    def handle(copies):
+        g = c.gauge(DIMS, U, "f64", 18)
+        assert g.nbytes == links * (2 if copies else 1)
+        assert rel(c.unpack(c.Qtm(g, c.empty(VH, "f64"), a, 0.16, 0.01), VH, "f64").cpu().numpy(), want) < 1e-13
+        return g
+
+    handle(True).close()
+    tmhop.tm_ctx_set_fixed_point(c.handle, False)
+    g = handle(False)
+    U_dev, n = tmhop._as_real_dev(U, c.device), tmhop.tm_gauge_storage_bytes(DIMS, tmhop.TM_F64, 18)
+    mem = torch.empty(n, dtype=torch.uint8, device=c.device)
+    h = tmhop.tm_gauge_create_in(c.handle, DIMS, U_dev, tmhop.TM_F64, 18, (-1, 1, 1, 1), mem, n)
+    assert tmhop.tm_gauge_bytes(h) == links
+    tmhop.tm_gauge_destroy(h)
+    tmhop.tm_ctx_set_fixed_point(c.handle, True)
+    handle(True).close()
+    free, total = torch.cuda.mem_get_info()
+    hold = torch.empty(free - total // 2 + (32 << 20), dtype=torch.uint8, device=c.device)   # less than half is left
+    handle(False).close()
+    del hold
+    torch.cuda.empty_cache()
+    handle(True).close()
+    g.close()
+    c.close()
