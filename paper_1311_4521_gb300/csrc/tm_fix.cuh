@@ -662,83 +662,6 @@ __device__ __forceinline__ float fx_narrow(double v, int e)
     return (hw | unsigned(__double2loint(v))) == 0u ? 0.f : r;
 }
 
-// The smallest nonzero sum of absolute products S that enters a component of
-// the hop at site i, in units of 2^e (infinite if all are zero), from the
-// FP64 input with FP64 projections; the products in single precision.
-template <int PR, int RECON, bool DAG> __device__ __forceinline__ float fx_least_sum(const FxArgs &A, unsigned i, int e)
-{
-    Nbrs n;
-    neighbours(A.g, A.p, i, n);
-    const GlobalLinks<F64, RECON> src{A.links, A.g.vh, i, A.p};
-    constexpr int SF = DAG ? +1 : -1, SB = -SF;
-    float sum[4][3][2] = {};
-#pragma unroll 1
-    for (int k = 0; k < 8; ++k) {
-        const int mu = k >> 1;
-        const bool fwd = (k & 1) == 0;
-        unsigned j = 0;
-#pragma unroll
-        for (int m = 0; m < 4; ++m)
-            if (m == mu) j = fwd ? n.fwd[m] : n.bwd[m];
-        Spinor<double> s;
-        Half<double> h;
-        Link<double> u;
-        SpinorIO<PR>::load_raw(A.exact, A.g.vh, j, s);
-        switch (k) {
-        case 0: project<0, SF>(s, h); src.template fwd<0>(n, u); break;
-        case 1: project<0, SB>(s, h); src.template bwd<0>(n, u); break;
-        case 2: project<1, SF>(s, h); src.template fwd<1>(n, u); break;
-        case 3: project<1, SB>(s, h); src.template bwd<1>(n, u); break;
-        case 4: project<2, SF>(s, h); src.template fwd<2>(n, u); break;
-        case 5: project<2, SB>(s, h); src.template bwd<2>(n, u); break;
-        case 6: project<3, SF>(s, h); src.template fwd<3>(n, u); break;
-        default: project<3, SB>(s, h); src.template bwd<3>(n, u); break;
-        }
-        float w[3][3][2], v[2][3][2];
-#pragma unroll
-        for (int a = 0; a < 3; ++a)
-#pragma unroll
-            for (int b = 0; b < 3; ++b) {
-                w[a][b][0] = fx_narrow(fwd ? u[a][b].re : u[b][a].re, 0);
-                w[a][b][1] = fx_narrow(fwd ? u[a][b].im : u[b][a].im, 0);
-            }
-#pragma unroll
-        for (int sp = 0; sp < 2; ++sp)
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                v[sp][c][0] = fx_narrow(h[sp][c].re, e);
-                v[sp][c][1] = fx_narrow(h[sp][c].im, e);
-            }
-        // the lower spin that an upper one feeds, and whether times i (fx_accumulate)
-        const bool cross = mu == 1 || mu == 2, times_i = mu == 1 || mu == 3;
-#pragma unroll
-        for (int sp = 0; sp < 2; ++sp)
-#pragma unroll
-            for (int a = 0; a < 3; ++a) {
-                float re = 0.f, im = 0.f;
-#pragma unroll
-                for (int b = 0; b < 3; ++b) {
-                    re += w[a][b][0] * v[sp][b][0] + w[a][b][1] * v[sp][b][1];
-                    im += w[a][b][0] * v[sp][b][1] + w[a][b][1] * v[sp][b][0];
-                }
-                sum[sp][a][0] += re;
-                sum[sp][a][1] += im;
-                const float x = times_i ? im : re, y = times_i ? re : im;
-                sum[2 + sp][a][0] += cross ? 0.f : x;
-                sum[2 + sp][a][1] += cross ? 0.f : y;
-                sum[3 - sp][a][0] += cross ? x : 0.f;
-                sum[3 - sp][a][1] += cross ? y : 0.f;
-            }
-    }
-    float least = __int_as_float(0x7f800000);
-#pragma unroll
-    for (int c = 0; c < 24; ++c) {
-        const float v = sum[c / 6][c / 2 % 3][c & 1];
-        if (v != 0.f) least = fminf(least, v);
-    }
-    return least;
-}
-
 // Whether the result of a fixed-point hop, o = a hop, may be stored in fixed
 // point (FxSite f), with `least` the smallest sum of absolute products of its
 // components in units of 2^e: FX_LEAST_STORED.
@@ -758,57 +681,134 @@ template <int P> __device__ __forceinline__ cpx<double> fx_load(const void *base
     return {v.x, v.y};
 }
 
-// fx_least_sum of one site by a whole warp: a lane takes one of the 8 hops,
-// one upper spin, and the real or the imaginary parts.
-template <int PR, int RECON, bool DAG> __device__ __forceinline__ float fx_least_sum_warp(const FxArgs &A, unsigned i, int e)
-{
-    using L = LinkIO<F64, RECON>;
-    constexpr unsigned all = 0xffffffffu;
-    const unsigned vh = A.g.vh, lane = threadIdx.x & 31;
-    const int k = lane & 7, mu = k >> 1, s = (lane >> 3) & 1, part = lane >> 4;
-    const bool fwd = (k & 1) == 0, cross = mu == 1 || mu == 2, times_i = mu == 1 || mu == 3;
-    Nbrs n;
-    neighbours(A.g, A.p, i, n);
-    unsigned j = 0, jb = 0;
-#pragma unroll
-    for (int m = 0; m < 4; ++m)
-        if (m == mu) {
-            j = fwd ? n.fwd[m] : n.bwd[m];
-            jb = fwd ? i : n.bwd[m];
-        }
+// One site by a whole warp: a lane takes one of the 8 hops, one upper spin s,
+// and the real or the imaginary parts.
+template <int PR, int RECON, bool DAG> struct FxWarpSite {
+    int k, mu, s, part;
+    bool fwd, cross, times_i, plus, neg;   // the lower spin that s feeds is 1 - s; times i; projector's sign; boundary
+    cpx<double> h[3];                      // the projected spin
     Link<double> u;
-    L::load(A.links + size_t(4 * (fwd ? A.p : 1 - A.p) + mu) * L::NCHUNK * vh, vh, jb, u);
-    // h_s = u_s + f l, f = 1, -1, i or -i (fx_project)
-    const bool plus = (DAG ? +1 : -1) * (fwd ? 1 : -1) > 0, toggle = mu < 2 || s == 0;
-    const double f = plus != toggle ? 1.0 : -1.0;
-    const int low = 2 + (cross ? 1 - s : s);
-    float v[3][2], x[3];
+    __device__ __forceinline__ FxWarpSite(const FxArgs &A, unsigned i)
+    {
+        using L = LinkIO<F64, RECON>;
+        const unsigned vh = A.g.vh, lane = threadIdx.x & 31;
+        k = lane & 7, mu = k >> 1, s = (lane >> 3) & 1, part = lane >> 4;
+        fwd = (k & 1) == 0, cross = mu == 1 || mu == 2, times_i = mu == 1 || mu == 3;
+        plus = (DAG ? +1 : -1) * (fwd ? 1 : -1) > 0;
+        Nbrs n;
+        neighbours(A.g, A.p, i, n);
+        unsigned j = 0, jb = 0;
+        neg = false;
+#pragma unroll
+        for (int m = 0; m < 4; ++m)
+            if (m == mu) {
+                j = fwd ? n.fwd[m] : n.bwd[m];
+                jb = fwd ? i : n.bwd[m];
+                neg = (fwd ? n.wf[m] : n.wb[m]) && A.g.anti[m];
+            }
+        L::load(A.links + size_t(4 * (fwd ? A.p : 1 - A.p) + mu) * L::NCHUNK * vh, vh, jb, u);
+        // h_s = u_s + f l, f = 1, -1, i or -i (fx_project)
+        const bool toggle = mu < 2 || s == 0;
+        const double f = plus != toggle ? 1.0 : -1.0;
+        const int low = 2 + (cross ? 1 - s : s);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const cpx<double> a = fx_load<PR>(A.exact, vh, j, 3 * s + c), l = fx_load<PR>(A.exact, vh, j, 3 * low + c);
+            h[c] = {a.re + f * (times_i ? -l.im : l.re), a.im + f * (times_i ? l.re : l.im)};
+        }
+    }
+    __device__ __forceinline__ cpx<double> link(int a, int b) const { return fwd ? u[a][b] : conj(u[b][a]); }
+    // The lane that holds this lane's share of a lower spin (and gives its own).
+    __device__ __forceinline__ int partner() const { return (cross ? 8 : 0) | (times_i ? 16 : 0); }
+};
+
+// The smallest nonzero sum of absolute products S that enters a component of
+// the hop at site i, in units of 2^e (infinite if all are zero), from the
+// FP64 input with FP64 projections; the products in single precision.
+template <int PR, int RECON, bool DAG> __device__ __forceinline__ float fx_least_sum(const FxArgs &A, unsigned i, int e)
+{
+    constexpr unsigned all = 0xffffffffu;
+    const FxWarpSite<PR, RECON, DAG> w(A, i);
+    float least = __int_as_float(0x7f800000), v[3][2];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        const cpx<double> a = fx_load<PR>(A.exact, vh, j, 3 * s + c), l = fx_load<PR>(A.exact, vh, j, 3 * low + c);
-        const float re = fx_narrow(a.re + f * (times_i ? -l.im : l.re), e), im = fx_narrow(a.im + f * (times_i ? l.re : l.im), e);
-        v[c][0] = part ? im : re;
-        v[c][1] = part ? re : im;
+        const float re = fx_narrow(w.h[c].re, e), im = fx_narrow(w.h[c].im, e);
+        v[c][0] = w.part ? im : re;
+        v[c][1] = w.part ? re : im;
     }
-    float least = __int_as_float(0x7f800000);
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        x[a] = 0.f;
+        float x = 0.f;
 #pragma unroll
-        for (int b = 0; b < 3; ++b)
-            x[a] += fx_narrow(fwd ? u[a][b].re : u[b][a].re, 0) * v[b][0] + fx_narrow(fwd ? u[a][b].im : u[b][a].im, 0) * v[b][1];
-        // the lower spin's share comes from the lane of the other spin or part where cross or times_i
-        float y = __shfl_xor_sync(all, x[a], int((cross ? 8u : 0u) | (times_i ? 16u : 0u)));
+        for (int b = 0; b < 3; ++b) x += fx_narrow(w.link(a, b).re, 0) * v[b][0] + fx_narrow(w.link(a, b).im, 0) * v[b][1];
+        float y = __shfl_xor_sync(all, x, w.partner());
 #pragma unroll
         for (int o = 1; o < 8; o *= 2) {
-            x[a] += __shfl_xor_sync(all, x[a], o);
+            x += __shfl_xor_sync(all, x, o);
             y += __shfl_xor_sync(all, y, o);
         }
-        if (x[a] != 0.f) least = fminf(least, x[a]);
+        if (x != 0.f) least = fminf(least, x);
         if (y != 0.f) least = fminf(least, y);
     }
     least = fminf(least, __shfl_xor_sync(all, least, 8));
     return fminf(least, __shfl_xor_sync(all, least, 16));
+}
+
+// Output site i with FP64 products, from the input to the stored result.
+// Returns whether all its hops are finite; if not, nothing is stored (the
+// order of the sums decides between NaN and infinities: fx_again's).
+template <int PR, int PX, int PO, int RECON, bool DAG, bool HASX>
+__device__ __forceinline__ bool fx_site_warp(const FxArgs &A, unsigned i)
+{
+    constexpr unsigned all = 0xffffffffu;
+    const unsigned vh = A.g.vh;
+    const FxWarpSite<PR, RECON, DAG> w(A, i);
+    double x[3], y[3];
+    bool finite = true;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        double r = 0.0;
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+            const cpx<double> u = w.link(a, b);
+            r += u.re * (w.part ? w.h[b].im : w.h[b].re);
+            r += u.im * (w.part ? w.h[b].re : -w.h[b].im);
+        }
+        x[a] = w.neg ? -r : r;
+        // as in accumulate(): what the lower spin gets of it, i r = (-im, re)
+        const int to = w.cross ? 1 - w.s : w.s;
+        bool minus = !w.plus;
+        if (w.mu == 0 || (w.mu >= 2 && to == 1)) minus = !minus;
+        if (w.times_i && w.part) minus = !minus;
+        y[a] = __shfl_xor_sync(all, minus ? -x[a] : x[a], w.partner());
+#pragma unroll
+        for (int o = 1; o < 8; o *= 2) {
+            x[a] += __shfl_xor_sync(all, x[a], o);
+            y[a] += __shfl_xor_sync(all, y[a], o);
+        }
+        finite = finite && fabs(x[a]) <= 1.7976931348623157e308 && fabs(y[a]) <= 1.7976931348623157e308;
+    }
+    if (!__all_sync(all, finite)) return false;
+    const int spin = (w.k == 0 ? 0 : 2) + w.s;   // of the lanes that store: parts re, hops 0 and 1
+    const bool up = spin < 2;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const double re = w.k == 0 ? x[a] : y[a], im = __shfl_xor_sync(all, re, 16);
+        if (w.part || w.k > 1) continue;
+        const cpx<double> hop = {re, im};
+        const double *d = A.k.d + (up ? 0 : 2);
+        cpx<double> o = A.k.unit ? (up ? hop : -hop) : cpx<double>{d[0], d[1]} * hop;
+        if (HASX) o = cmadd(cpx<double>{d[4], d[5]}, fx_load<PX>(A.x, vh, i, 3 * spin + a), o);
+        const int c = 3 * spin + a;
+        if (PO == FXF) {
+            st_stream(fx_entry(static_cast<int4 *>(A.out), FX_SPINOR_BLOCK, i) + 32 * c,
+                      make_int4(__double2hiint(o.re), __double2loint(o.re), __double2hiint(o.im), __double2loint(o.im)));
+            if (c == 0) st_stream(const_cast<int *>(fx_words(A.out, vh)) + i, FX_RAW);
+        } else {
+            st_stream(static_cast<double2 *>(A.out) + (PO == F64C ? size_t(i) * 12 + c : size_t(c) * vh + i), make_double2(o.re, o.im));
+        }
+    }
+    return true;
 }
 
 // What is left to do at output site i after its fixed-point hop.
@@ -819,39 +819,49 @@ enum { FX_DONE = 0, FX_CHECK = 1, FX_SLOW = 2 };
 // sum of absolute products is large enough (for a fixed-point output also for
 // it to be stored so).  FX_SLOW and the others: computed with FP64 products,
 // from the input to the stored result.  A call whose arguments are few words:
-// passing the site's sum in and out cost 7 % of the kernel.  Up to 4 sites are
-// checked by the whole warp: alone, a lane's 8 hops are a chain of several us
-// that every launch had to wait for somewhere (Q_tm on 16^4 69 us, now 40; on
-// 8^4 45, now 16); more of them (a field with components of exactly zero) by
-// a lane each.
+// passing the site's sum in and out cost 7 % of the kernel.
+// Up to FX_FEW sites are done one by one by the whole warp.  By a lane each,
+// the check was a chain of several us that every launch waited for somewhere
+// (Q_tm on 16^4 69 us, now 40; on 8^4 45, now 16), and FP64 products a longer
+// one (16^4, unit links, with such sites: 113 us, now 73).  With 16 a point
+// source on 8^4 took 95 us against 84.  More of them are not checked: they
+// come from fields of graded components, for which the check is spent in vain
+// (Q_tm on 24^3x48, all sites: 1.60 ms with, 1.44 without; 1.02 with FP64
+// products alone).
+constexpr int FX_FEW = 8;
 template <int PR, int PX, int PO, int RECON, bool DAG, bool HASX>
 __device__ __noinline__ void fx_again(const FxArgs &A, unsigned i, int e, int todo)
 {
     constexpr unsigned all = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    __syncwarp();   // results stored so far come before what other lanes replace
     unsigned check = __ballot_sync(all, todo == FX_CHECK);
-    float least = 0.f;
-    if (__popc(check) > 4) {
-        if (todo == FX_CHECK) least = fx_least_sum<PR, RECON, DAG>(A, i, e);
-    } else {
+    if (__popc(check) <= FX_FEW) {
         while (check) {
-            const int lane = __ffs(int(check)) - 1;
+            const int q = __ffs(int(check)) - 1;
             check &= check - 1;
-            const float of_lane = fx_least_sum_warp<PR, RECON, DAG>(A, __shfl_sync(all, i, lane), __shfl_sync(all, e, lane));
-            if (int(threadIdx.x & 31) == lane) least = of_lane;
+            const float least = fx_least_sum<PR, RECON, DAG>(A, __shfl_sync(all, i, q), __shfl_sync(all, e, q));
+            if (lane != q) continue;
+            bool stays = least >= float(FX_LEAST);
+            if (PO == FXF) {
+                const int word = static_cast<const volatile int *>(fx_words(A.out, A.g.vh))[i];
+                FxSite f(0, 0);
+                f.raw = word == FX_RAW;
+                f.e = int(short(word & 0xffff));
+                stays = stays && fx_stores(A, least, e, f);
+            }
+            if (stays) todo = FX_DONE;
+        }
+    }
+    unsigned slow = __ballot_sync(all, todo != FX_DONE);
+    if (__popc(slow) <= FX_FEW) {
+        while (slow) {
+            const int q = __ffs(int(slow)) - 1;
+            slow &= slow - 1;
+            if (fx_site_warp<PR, PX, PO, RECON, DAG, HASX>(A, __shfl_sync(all, i, q)) && lane == q) todo = FX_DONE;
         }
     }
     if (todo == FX_DONE) return;
-    if (todo == FX_CHECK) {
-        bool stays = least >= float(FX_LEAST);
-        if (PO == FXF) {
-            const int word = static_cast<const volatile int *>(fx_words(A.out, A.g.vh))[i];
-            FxSite f(0, 0);
-            f.raw = word == FX_RAW;
-            f.e = int(short(word & 0xffff));
-            stays = stays && fx_stores(A, least, e, f);
-        }
-        if (stays) return;
-    }
     Nbrs n;
     neighbours(A.g, A.p, i, n);
     GlobalLinks<F64, RECON> src{A.links, A.g.vh, i, A.p};
@@ -944,6 +954,7 @@ __device__ __forceinline__ bool fx_finish(const FxArgs &A, unsigned i, bool on, 
     }
     if (!__any_sync(0xffffffffu, todo != FX_DONE)) return false;
     fx_again<PR, PX, PO, RECON, DAG, HASX>(A, i, v.e, todo);
+    __syncwarp();   // a site may have been stored by other lanes than its own
     return true;
 }
 
