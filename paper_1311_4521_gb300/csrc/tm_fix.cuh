@@ -681,6 +681,83 @@ template <int P> __device__ __forceinline__ cpx<double> fx_load(const void *base
     return {v.x, v.y};
 }
 
+// The smallest nonzero sum of absolute products S that enters a component of
+// the hop at site i, in units of 2^e (infinite if all are zero), from the
+// FP64 input with FP64 projections; the products in single precision.
+template <int PR, int RECON, bool DAG> __device__ __forceinline__ float fx_least_sum(const FxArgs &A, unsigned i, int e)
+{
+    Nbrs n;
+    neighbours(A.g, A.p, i, n);
+    const GlobalLinks<F64, RECON> src{A.links, A.g.vh, i, A.p};
+    constexpr int SF = DAG ? +1 : -1, SB = -SF;
+    float sum[4][3][2] = {};
+#pragma unroll 1
+    for (int k = 0; k < 8; ++k) {
+        const int mu = k >> 1;
+        const bool fwd = (k & 1) == 0;
+        unsigned j = 0;
+#pragma unroll
+        for (int m = 0; m < 4; ++m)
+            if (m == mu) j = fwd ? n.fwd[m] : n.bwd[m];
+        Spinor<double> s;
+        Half<double> h;
+        Link<double> u;
+        SpinorIO<PR>::load_raw(A.exact, A.g.vh, j, s);
+        switch (k) {
+        case 0: project<0, SF>(s, h); src.template fwd<0>(n, u); break;
+        case 1: project<0, SB>(s, h); src.template bwd<0>(n, u); break;
+        case 2: project<1, SF>(s, h); src.template fwd<1>(n, u); break;
+        case 3: project<1, SB>(s, h); src.template bwd<1>(n, u); break;
+        case 4: project<2, SF>(s, h); src.template fwd<2>(n, u); break;
+        case 5: project<2, SB>(s, h); src.template bwd<2>(n, u); break;
+        case 6: project<3, SF>(s, h); src.template fwd<3>(n, u); break;
+        default: project<3, SB>(s, h); src.template bwd<3>(n, u); break;
+        }
+        float w[3][3][2], v[2][3][2];
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+#pragma unroll
+            for (int b = 0; b < 3; ++b) {
+                w[a][b][0] = fx_narrow(fwd ? u[a][b].re : u[b][a].re, 0);
+                w[a][b][1] = fx_narrow(fwd ? u[a][b].im : u[b][a].im, 0);
+            }
+#pragma unroll
+        for (int sp = 0; sp < 2; ++sp)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                v[sp][c][0] = fx_narrow(h[sp][c].re, e);
+                v[sp][c][1] = fx_narrow(h[sp][c].im, e);
+            }
+        // the lower spin that an upper one feeds, and whether times i (fx_accumulate)
+        const bool cross = mu == 1 || mu == 2, times_i = mu == 1 || mu == 3;
+#pragma unroll
+        for (int sp = 0; sp < 2; ++sp)
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                float re = 0.f, im = 0.f;
+#pragma unroll
+                for (int b = 0; b < 3; ++b) {
+                    re += w[a][b][0] * v[sp][b][0] + w[a][b][1] * v[sp][b][1];
+                    im += w[a][b][0] * v[sp][b][1] + w[a][b][1] * v[sp][b][0];
+                }
+                sum[sp][a][0] += re;
+                sum[sp][a][1] += im;
+                const float x = times_i ? im : re, y = times_i ? re : im;
+                sum[2 + sp][a][0] += cross ? 0.f : x;
+                sum[2 + sp][a][1] += cross ? 0.f : y;
+                sum[3 - sp][a][0] += cross ? x : 0.f;
+                sum[3 - sp][a][1] += cross ? y : 0.f;
+            }
+    }
+    float least = __int_as_float(0x7f800000);
+#pragma unroll
+    for (int c = 0; c < 24; ++c) {
+        const float v = sum[c / 6][c / 2 % 3][c & 1];
+        if (v != 0.f) least = fminf(least, v);
+    }
+    return least;
+}
+
 // One site by a whole warp: a lane takes one of the 8 hops, one upper spin s,
 // and the real or the imaginary parts.
 template <int PR, int RECON, bool DAG> struct FxWarpSite {
@@ -722,10 +799,8 @@ template <int PR, int RECON, bool DAG> struct FxWarpSite {
     __device__ __forceinline__ int partner() const { return (cross ? 8 : 0) | (times_i ? 16 : 0); }
 };
 
-// The smallest nonzero sum of absolute products S that enters a component of
-// the hop at site i, in units of 2^e (infinite if all are zero), from the
-// FP64 input with FP64 projections; the products in single precision.
-template <int PR, int RECON, bool DAG> __device__ __forceinline__ float fx_least_sum(const FxArgs &A, unsigned i, int e)
+// fx_least_sum of one site by a whole warp.
+template <int PR, int RECON, bool DAG> __device__ __forceinline__ float fx_least_sum_warp(const FxArgs &A, unsigned i, int e)
 {
     constexpr unsigned all = 0xffffffffu;
     const FxWarpSite<PR, RECON, DAG> w(A, i);
@@ -821,13 +896,16 @@ enum { FX_DONE = 0, FX_CHECK = 1, FX_SLOW = 2 };
 // from the input to the stored result.  A call whose arguments are few words:
 // passing the site's sum in and out cost 7 % of the kernel.
 // Up to FX_FEW sites are done one by one by the whole warp.  By a lane each,
-// the check was a chain of several us that every launch waited for somewhere
+// the check is a chain of several us that every launch waited for somewhere
 // (Q_tm on 16^4 69 us, now 40; on 8^4 45, now 16), and FP64 products a longer
 // one (16^4, unit links, with such sites: 113 us, now 73).  With 16 a point
-// source on 8^4 took 95 us against 84.  More of them are not checked: they
-// come from fields of graded components, for which the check is spent in vain
-// (Q_tm on 24^3x48, all sites: 1.60 ms with, 1.44 without; 1.02 with FP64
-// products alone).
+// source on 8^4 took 95 us against 84.  More are checked and computed by a
+// lane each: checks one by one take 35 us per site of a warp and launch on
+// 24^3x48, by all lanes at once 80.  Such fields have components of exactly
+// zero, which only the check tells from small ones (Q_tm on a field of one
+// spin, 24^3x48, links exp(0.3 i A): 1.45 ms unchecked, 0.45 checked), or
+// components of very different size, for which it is spent in vain (1.58
+// against 1.45 ms; 1.02 with FP64 products throughout).
 constexpr int FX_FEW = 8;
 template <int PR, int PX, int PO, int RECON, bool DAG, bool HASX>
 __device__ __noinline__ void fx_again(const FxArgs &A, unsigned i, int e, int todo)
@@ -836,22 +914,28 @@ __device__ __noinline__ void fx_again(const FxArgs &A, unsigned i, int e, int to
     const int lane = threadIdx.x & 31;
     __syncwarp();   // results stored so far come before what other lanes replace
     unsigned check = __ballot_sync(all, todo == FX_CHECK);
-    if (__popc(check) <= FX_FEW) {
+    float least = 0.f;
+    if (__popc(check) > FX_FEW) {
+        if (todo == FX_CHECK) least = fx_least_sum<PR, RECON, DAG>(A, i, e);
+        __syncwarp();
+    } else {
         while (check) {
             const int q = __ffs(int(check)) - 1;
             check &= check - 1;
-            const float least = fx_least_sum<PR, RECON, DAG>(A, __shfl_sync(all, i, q), __shfl_sync(all, e, q));
-            if (lane != q) continue;
-            bool stays = least >= float(FX_LEAST);
-            if (PO == FXF) {
-                const int word = static_cast<const volatile int *>(fx_words(A.out, A.g.vh))[i];
-                FxSite f(0, 0);
-                f.raw = word == FX_RAW;
-                f.e = int(short(word & 0xffff));
-                stays = stays && fx_stores(A, least, e, f);
-            }
-            if (stays) todo = FX_DONE;
+            const float of_q = fx_least_sum_warp<PR, RECON, DAG>(A, __shfl_sync(all, i, q), __shfl_sync(all, e, q));
+            if (lane == q) least = of_q;
         }
+    }
+    if (todo == FX_CHECK) {
+        bool stays = least >= float(FX_LEAST);
+        if (PO == FXF) {
+            const int word = static_cast<const volatile int *>(fx_words(A.out, A.g.vh))[i];
+            FxSite f(0, 0);
+            f.raw = word == FX_RAW;
+            f.e = int(short(word & 0xffff));
+            stays = stays && fx_stores(A, least, e, f);
+        }
+        if (stays) todo = FX_DONE;
     }
     unsigned slow = __ballot_sync(all, todo != FX_DONE);
     if (__popc(slow) <= FX_FEW) {

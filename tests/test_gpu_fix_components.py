@@ -163,3 +163,35 @@ def test_host_fields_give_the_same_bits(ctx, lattice, kind):
     ctx.Qtm_host(g, [o], [a], KAPPA, MU)
     assert np.array_equal(o.numpy(), apply(ctx, g, psi, "qtm", KAPPA, MU))
     g.close()
+
+
+@pytest.mark.parametrize("lattice,recon", [(SMALL, 18), (SMALL, 12), (LARGE, 18)])
+@pytest.mark.parametrize("links,keep", [("near", "spin"), ("near", "spin, real"), ("unit", "spin"), ("unit", "component"),
+                                        ("diagonal", "component"), ("real", "colour, real")])
+def test_exact_zeros_stay_with_the_integers(ctx, lattice, recon, links, keep):
+    """Fields diluted in spin and colour: components that nothing but zeros enters do not send their sites to FP64
+    products.  Those would give the bits of a handle without a fixed-point copy at every site; the integers round some
+    sums the other way (unit links, real fields: few of the nonzero components' sums are rounded at all)."""
+    from paper_1311_4521_gb300 import tmhop
+    dims, bc = lattice
+    U, psi = gauge(dims, links), field(dims, "gauss")
+    if recon == 12:
+        U[..., 2, :] = np.cross(U[..., 0, :], U[..., 1, :]).conj()
+    if "real" in keep:
+        psi = psi.real + 0j
+    if "spin" in keep or "component" in keep:
+        psi[:, (0, 1, 3)] = 0
+    if "colour" in keep or "component" in keep:
+        psi[..., (0, 2)] = 0
+    E = Absolute(dims, U, bc)
+    g = ctx.gauge(dims, U, "f64", recon, bc)
+    tmhop.tm_ctx_set_fixed_point(ctx.handle, False)
+    products = ctx.gauge(dims, U, "f64", recon, bc)
+    tmhop.tm_ctx_set_fixed_point(ctx.handle, True)
+    got = apply(ctx, g, psi, (1, False))
+    assert within(got, E.hop(psi, 1, False), E.sums(psi, 1, False))
+    assert not np.array_equal(got, apply(ctx, products, psi, (1, False)))
+    if lattice is SMALL:
+        assert within(apply(ctx, g, psi, "qtm", KAPPA, MU), E.qtm(psi, KAPPA, MU), E.qtm_bound(psi, KAPPA, MU))
+    products.close()
+    g.close()
