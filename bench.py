@@ -59,25 +59,28 @@ def fp64_nominal_tflops(sm_count: int, sm_mhz: float) -> float:
 # DRAM bytes (read + write) per launch of Q_tm's launch B from ncu captures of
 # the dominant kernel on the 32^3x64 workload lattice (per site, so that
 # another lattice scales by its site count), valid only for the kernel
-# sources they were taken from (hash of csrc/tm_device.cuh +
-# csrc/tm_kernels.cu).
-TRAFFIC = {"src": "4d1e82678e27f879",
-           "per_site": {("f64", 18): 1790570752 / 1048576, ("f64x", 18): 1790290944 / 1048576,
-                        ("f32", 12): 678930688 / 1048576, ("f16", 12): 341252096 / 1048576}}
+# sources they were taken from.  FP64 with fixed-point links (k_fx_hop) and
+# with FP64 products (k_hop) are different kernels; the second has no capture
+# of these sources.
+TRAFFIC_SOURCES = ("tm_device.cuh", "tm_kernels.cu", "tm_fix.cuh", "tm_fix.cu")
+TRAFFIC = {"src": "deba072047ea63b8",
+           "per_site": {("f64", 18): 1918322688 / 1048576, ("f64x", 18): 1790149120 / 1048576,
+                        ("f32", 12): 695441408 / 1048576, ("f16", 12): 347103488 / 1048576}}
 
 
 def kernel_source_hash() -> str:
     import hashlib
     h = hashlib.sha256()
-    for f in ("tm_device.cuh", "tm_kernels.cu"):
+    for f in TRAFFIC_SOURCES:
         with open(os.path.join(ROOT, "paper_1311_4521_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
 
 
-def traffic_per_launch(prec: str, recon: int, vh: int):
+def traffic_per_launch(prec: str, recon: int, vh: int, fixed: bool = True):
+    """None for FP64 handles without fixed-point links (fixed False)."""
     per = TRAFFIC["per_site"].get((prec, recon))
-    if per is None or kernel_source_hash() != TRAFFIC["src"]:
+    if per is None or (prec == "f64" and not fixed) or kernel_source_hash() != TRAFFIC["src"]:
         return None
     return round(per * vh)
 
@@ -320,13 +323,13 @@ def gpu_arm(args) -> None:
     gflops = world * vh * QTM_FLOPS / (ms_per_step * 1e-3) / 1e9
     kb_tflops = vh * (HOP_FLOPS + 96) / (kb_ms * 1e-3) / 1e12
     kb_gbs = vh * ab["kernel_b"] / (kb_ms * 1e-3) / 1e9
-    traffic = args.traffic if args.traffic is not None else traffic_per_launch(prec, recon, vh)
     kname = f"k_hop<{prec.upper()},{recon},HASX> (Q_tm second launch: H_eo + gamma5 twisted update)"
     fixed = prec == "f64" and tmhop.tm_gauge_bytes(g.handle) > 8 * vh * 8 * recon   # links also in fixed point
+    traffic = args.traffic if args.traffic is not None else traffic_per_launch(prec, recon, vh, fixed)
     if fixed:   # link products on the integer units: bound by memory and those, no longer by the FP64 pipe
         kname = f"k_fx_hop<F64,{recon},HASX> (Q_tm second launch: H_eo + gamma5 twisted update)"
         roofline = {"bound": "hbm", "achieved": round(kb_gbs, 1), "peak": hbm_peak, "unit": "GB/s",
-                    "frac": round(kb_gbs / hbm_peak, 4), "traffic": args.traffic, "kernel": kname,
+                    "frac": round(kb_gbs / hbm_peak, 4), "traffic": traffic, "kernel": kname,
                     "peak_source": f"{hbm_src} HBM copy bandwidth", "tflops": round(kb_tflops, 4),
                     "fp64_pipe_peak_tflops": round(fp64_peak, 4)}
     elif prec == "f64":
